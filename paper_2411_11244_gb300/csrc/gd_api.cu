@@ -955,7 +955,7 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
         const int cur = sort_points(g, ctx->pkeys, ctx->pvals, ctx->phist, ctx->stream);
         g.order = ctx->pvals[cur];
     }
-    GD_CUDA(ctx, launch_point(g, ctx->stream));
+    GD_CUDA(ctx, launch_point(g, ctx->sms, ctx->stream));
     if (!dev_out)
         GD_CUDA(ctx, cudaMemcpyAsync(out, ctx->pres_dev, sizeof(gd_point_result) * n, cudaMemcpyDeviceToHost, ctx->stream));
     unsigned long long w[kPointWords];

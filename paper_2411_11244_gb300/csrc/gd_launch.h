@@ -78,7 +78,8 @@ enum : int {
     kPointExact = 1,     // float64 point-triangle distances
     kPointT0 = 2,        // globaltimer stamp of the first CTA to start
     kPointTimeout = 3,   // some point passed the deadline
-    kPointWords = 4,
+    kPointTicket = 4,    // points handed out to warps
+    kPointWords = 8,
 };
 
 struct PointArgs {
@@ -90,7 +91,7 @@ struct PointArgs {
     const double* pts;    // n x 3 world points, device
     long long n;
     gd_point_result* out; // n results, device
-    const unsigned* order;// thread i answers point order[i] (nullptr: point i)
+    const unsigned* order;// order of work: the i-th point taken is order[i] (nullptr: point i)
     unsigned long long* ws;
     long long timeout_ns;
 };
@@ -100,7 +101,8 @@ struct PointArgs {
 // [returned index]; hist: build_hist_words(n) words
 int sort_points(const PointArgs& g, unsigned long long* const keys[2], unsigned* const vals[2], unsigned* hist,
                 cudaStream_t stream);
-cudaError_t launch_point(const PointArgs& g, cudaStream_t stream);
+// sms: the device's SM count
+cudaError_t launch_point(const PointArgs& g, int sms, cudaStream_t stream);
 
 // ---- query (gd_query.cu)
 // co-resident CTAs per SM of the query kernel's single-query or batch launch

@@ -951,6 +951,62 @@ def test_point_distance_device_io_and_edges(G, ctx, oracle_mod):
         G.gd_mesh_destroy(h)
 
 
+@pytest.mark.parametrize("T", [1, 2, 3, 31, 32, 33, 63, 64, 65, 127, 128, 255, 511, 1023, 2048])
+def test_point_walk_tree_depths(G, ctx, oracle_mod, T):
+    """Trees of 0 to 11 levels (the root's first step takes 0 to 5 of them,
+    the others three each), 1 to 67 points (part of a warp, more than one)."""
+    rng = np.random.default_rng(100 + T)
+    m = _soup(rng, T, 0.7)
+    h = _mesh(G, ctx, m)
+    try:
+        for n in (1, 2, 31, 33, 67):
+            x = _rigid(rng)
+            pts = rng.permutation(_probe_points(rng, m, x, n))[:n]
+            check_points(G.gd_point_distance(ctx, h, x, pts), m, x, pts, oracle_mod)
+    finally:
+        G.gd_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("copies", [31, 32, 33, 64, 200])
+def test_point_ties_take_the_smallest_index(G, ctx, oracle_mod, copies):
+    """Many copies of each triangle: more candidates at one distance than a
+    warp holds; the answer is the first copy.  A point beyond float32's range
+    (every float32 bound infinite) is still answered in float64."""
+    rng = np.random.default_rng(200 + copies)
+    v, t = _soup(rng, 7, 0.7)
+    m = (v, np.tile(t, (copies, 1)))
+    h = _mesh(G, ctx, m)
+    try:
+        x = _rigid(rng)
+        pts = _probe_points(rng, m, x, 40)
+        r = G.gd_point_distance(ctx, h, x, pts)
+        check_points(r, m, x, pts, oracle_mod)
+        assert (r["tri"] < 7).all()
+        far = np.array([[1e40, 0.0, 0.0], [0.0, -3e60, 1e60]])
+        r = G.gd_point_distance(ctx, h, x, far)
+        assert list(r["status"]) == [0, 0]
+        assert np.allclose(r["d"], np.linalg.norm(far, axis=1), rtol=1e-14, atol=0)
+    finally:
+        G.gd_mesh_destroy(h)
+
+
+def test_point_order_and_caller_order_agree(G, ctx):
+    """Calls of 2^14 points and more are walked along a Morton curve; the same
+    points in small calls are not: the records are the same bits."""
+    rng = np.random.default_rng(61)
+    m = synth.torus(1.0, 0.05, 250, 30)
+    h = _mesh(G, ctx, m)
+    try:
+        x = _rigid(rng)
+        pts = _probe_points(rng, m, x, (1 << 14) + 5)
+        whole = G.gd_point_distance(ctx, h, x, pts)
+        parts = np.concatenate([G.gd_point_distance(ctx, h, x, p) for p in np.array_split(pts, 7)])
+        for f in ("d", "tri", "p", "status"):
+            assert np.array_equal(whole[f], parts[f])
+    finally:
+        G.gd_mesh_destroy(h)
+
+
 # ------------------------------------------------------------------ naive comparator
 
 def test_naive_comparator_matches_oracle(G, ctx, oracle_mod):
