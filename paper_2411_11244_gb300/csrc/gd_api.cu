@@ -89,6 +89,8 @@ struct gd_ctx {
     long long cap_ftree = 0;      // ... its capacity in nodes
     unsigned long long* naive_ws = nullptr;  // scratch of the naive comparator
     unsigned long long* point_ws = nullptr;  // counters of point queries
+    char* point_share = nullptr;             // ... and the room for shared walks
+    unsigned point_epoch = 0;
     double* pts_dev = nullptr;               // staged host points and results
     gd_point_result* pres_dev = nullptr;
     long long cap_pts = 0;
@@ -574,7 +576,7 @@ GD_API void gd_ctx_destroy(gd_ctx* c) {
     cudaFree(c->slot_of);
     cudaFree(c->ftree);
     cudaFree(c->naive_ws);
-    cudaFree(c->point_ws); cudaFree(c->pts_dev); cudaFree(c->pres_dev);
+    cudaFree(c->point_ws); cudaFree(c->point_share); cudaFree(c->pts_dev); cudaFree(c->pres_dev);
     cudaFree(c->pkeys[0]); cudaFree(c->pkeys[1]); cudaFree(c->pvals[0]); cudaFree(c->pvals[1]);
     cudaFree(c->phist);
     cudaStreamDestroy(c->stream);
@@ -916,6 +918,10 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
     if (n == 0) return GD_OK;
     cudaSetDevice(ctx->device);
     if (!ctx->point_ws) GD_CUDA(ctx, cudaMalloc(&ctx->point_ws, sizeof(unsigned long long) * kPointWords));
+    if (!ctx->point_share) {
+        GD_CUDA(ctx, cudaMalloc(&ctx->point_share, kPointShareBytes));
+        GD_CUDA(ctx, cudaMemsetAsync(ctx->point_share, 0, kPointShareBytes, ctx->stream));
+    }
     const bool dev_in = on_device(points), dev_out = on_device(out);
     if ((!dev_in || !dev_out) && n > ctx->cap_pts) {
         cudaFree(ctx->pts_dev); cudaFree(ctx->pres_dev);
@@ -932,6 +938,11 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
     g.out = dev_out ? out : ctx->pres_dev;
     g.ws = ctx->point_ws;
     g.timeout_ns = ctx->tun.timeout_ns;
+    if (++ctx->point_epoch == 0) ctx->point_epoch = 1;  // 0: never written
+    g.epoch = ctx->point_epoch;
+    g.shares = reinterpret_cast<PointShare*>(ctx->point_share);
+    g.parts = reinterpret_cast<PointPart*>(g.shares + kPointMaxShares);
+    g.slots = reinterpret_cast<PointSlot*>(g.parts + kPointMaxSlots + kPointMaxShares);
     if (!dev_in)
         GD_CUDA(ctx, cudaMemcpyAsync(ctx->pts_dev, points, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
     // enough points to fill the GPU: walk them in Morton order (warps of
@@ -963,7 +974,7 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
     GD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->last_point_tests = w[kPointTests];
     ctx->last_point_exact = w[kPointExact];
-    if (w[kPointTimeout]) return fail(ctx, GD_ERR_TIMEOUT, "a point query passed the timeout");
+    if (w[kPointTimeout] || w[kPointAnswered] < (unsigned long long)n) return fail(ctx, GD_ERR_TIMEOUT, "a point query passed the timeout");
     return GD_OK;
 }
 

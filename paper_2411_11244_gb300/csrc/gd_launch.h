@@ -78,9 +78,46 @@ enum : int {
     kPointExact = 1,     // float64 point-triangle distances
     kPointT0 = 2,        // globaltimer stamp of the first CTA to start
     kPointTimeout = 3,   // some point passed the deadline
-    kPointTicket = 4,    // points handed out to warps
-    kPointWords = 8,
+    kPointSlots = 4,     // points whose walk is shared
+    kPointParts = 5,     // answers of parts of shared walks
+    // (words that all warps use, a 128-byte line each)
+    kPointTicket = 16,   // points handed out to warps
+    kPointHead = 32,     // gifts claimed by idle warps
+    kPointTail = 48,     // gifts made
+    kPointAnswered = 64, // points answered
+    kPointWords = 80,
 };
+
+// Shared walks: a warp with a long walk gives parts of its stack to idle
+// warps.  Fixed room, reused by every call; when it is full walks are no longer
+// divided.
+constexpr unsigned kPointMaxSlots = 1u << 14;   // points with a shared walk
+constexpr unsigned kPointMaxShares = 1u << 16;  // gifts
+
+struct PointSlot {
+    unsigned U;       // least upper bound of all parts (float bits, squared)
+    unsigned parts;   // parts still running
+    unsigned chain;   // latest answer of a part (index into parts, kNone: none)
+    unsigned i;       // the point
+    unsigned failed;  // a part ran into the deadline
+};
+
+struct PointShare {
+    unsigned ready;   // the call's epoch once the gift is complete
+    unsigned slot, n, pad;
+    unsigned node[32];
+};
+
+constexpr unsigned kPartCands = 6;
+
+struct PointPart {
+    unsigned n, next;
+    unsigned tri[kPartCands];
+    float low[kPartCands];
+};
+
+constexpr size_t kPointShareBytes = sizeof(PointShare) * kPointMaxShares + sizeof(PointSlot) * kPointMaxSlots +
+                                    sizeof(PointPart) * (kPointMaxSlots + kPointMaxShares);
 
 struct PointArgs {
     const float* box;     // the mesh's tree
@@ -94,6 +131,12 @@ struct PointArgs {
     const unsigned* order;// order of work: the i-th point taken is order[i] (nullptr: point i)
     unsigned long long* ws;
     long long timeout_ns;
+    unsigned epoch;       // differs from call to call
+    unsigned share_steps; // steps of a walk before it gives any of it away (set by launch_point),
+    unsigned share_mask;  //   looks for idle warps in steps whose low bits these are zero
+    PointShare* shares;   // kPointMaxShares
+    PointSlot* slots;     // kPointMaxSlots
+    PointPart* parts;     // kPointMaxSlots + kPointMaxShares
 };
 
 // order the points along a Morton curve in the mesh's frame so that a warp's
@@ -102,7 +145,7 @@ struct PointArgs {
 int sort_points(const PointArgs& g, unsigned long long* const keys[2], unsigned* const vals[2], unsigned* hist,
                 cudaStream_t stream);
 // sms: the device's SM count
-cudaError_t launch_point(const PointArgs& g, int sms, cudaStream_t stream);
+cudaError_t launch_point(PointArgs g, int sms, cudaStream_t stream);
 
 // ---- query (gd_query.cu)
 // co-resident CTAs per SM of the query kernel's single-query or batch launch
