@@ -96,7 +96,7 @@ struct gd_ctx {
     long long cap_pts = 0;
     unsigned long long* pkeys[2] = {nullptr, nullptr};  // Morton ordering of the points
     unsigned* pvals[2] = {nullptr, nullptr};
-    unsigned* phist = nullptr;
+    void* psort = nullptr;
     long long cap_psort = 0;
     unsigned long long last_point_tests = 0, last_point_exact = 0;  // counters of the last point call
     gd_stats last{};
@@ -578,7 +578,7 @@ GD_API void gd_ctx_destroy(gd_ctx* c) {
     cudaFree(c->naive_ws);
     cudaFree(c->point_ws); cudaFree(c->point_share); cudaFree(c->pts_dev); cudaFree(c->pres_dev);
     cudaFree(c->pkeys[0]); cudaFree(c->pkeys[1]); cudaFree(c->pvals[0]); cudaFree(c->pvals[1]);
-    cudaFree(c->phist);
+    cudaFree(c->psort);
     cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -760,7 +760,9 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     GD_ALLOC(b.keys[1], sizeof(unsigned long long) * m->nt);
     GD_ALLOC(b.vals[0], sizeof(unsigned) * m->nt);
     GD_ALLOC(b.vals[1], sizeof(unsigned) * m->nt);
-    GD_ALLOC(b.hist, sizeof(unsigned) * build_hist_words(m->nt));
+    void* sort_mem = nullptr;
+    GD_ALLOC(sort_mem, sort_scratch_bytes(m->nt));
+    b.sort = sort_scratch(sort_mem, m->nt);
 #undef GD_ALLOC
     cudaError_t e = cudaMalloc(&m->d_box, sizeof(float) * 6 * (2ull << L));
     if (e == cudaSuccess) e = cudaMalloc(&m->d_tri, sizeof(float4) * 3 * m->nt);
@@ -786,12 +788,24 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     if (flags[0]) { drop_events(); cleanup(); return fail(ctx, GD_ERR_INVALID_ARG, "triangle index out of range"); }
     if (flags[1]) { drop_events(); cleanup(); return fail(ctx, GD_ERR_INVALID_ARG, "non-finite vertex coordinate"); }
     cudaEventRecord(ev[2], ctx->stream);
-    e = build_tree(b, ctx->stream);
-    cudaEventRecord(ev[3], ctx->stream);
     float root[6];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(root, m->d_box + 6, sizeof(root), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    unsigned ties = 0, sort_err = 0;
+    for (int all_bits = 0; all_bits < 2 && e == cudaSuccess; ++all_bits) {
+        e = build_tree(b, all_bits != 0, ctx->stream);
+        cudaEventRecord(ev[3], ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(root, m->d_box + 6, sizeof(root), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&ties, b.flags + kFlagTies, sizeof(ties), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&sort_err, b.sort.err, sizeof(sort_err), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        if (!ties) break;
+    }
     cleanup();
+    if (e == cudaSuccess && sort_err) {
+        drop_events();
+        return fail(ctx, GD_ERR_TIMEOUT, "a device-side wait of the build's sort timed out");
+    }
     if (e == cudaSuccess) {
         float t0 = 0.f, t1 = 0.f;
         cudaEventElapsedTime(&t0, ev[0], ev[1]);
@@ -953,18 +967,20 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
                 cudaFree(ctx->pkeys[k]); cudaFree(ctx->pvals[k]);
                 ctx->pkeys[k] = nullptr; ctx->pvals[k] = nullptr;
             }
-            cudaFree(ctx->phist);
-            ctx->phist = nullptr;
+            cudaFree(ctx->psort);
+            ctx->psort = nullptr;
             ctx->cap_psort = 0;
             for (int k = 0; k < 2; ++k) {
                 GD_CUDA(ctx, cudaMalloc(&ctx->pkeys[k], sizeof(unsigned long long) * n));
                 GD_CUDA(ctx, cudaMalloc(&ctx->pvals[k], sizeof(unsigned) * n));
             }
-            GD_CUDA(ctx, cudaMalloc(&ctx->phist, sizeof(unsigned) * build_hist_words(n)));
+            GD_CUDA(ctx, cudaMalloc(&ctx->psort, std::max(sort_scratch_bytes(n), sort_scratch_bytes(1ll << 18))));
             ctx->cap_psort = n;
         }
-        const int cur = sort_points(g, ctx->pkeys, ctx->pvals, ctx->phist, ctx->stream);
+        const SortWork w = sort_scratch(ctx->psort, n);
+        const int cur = sort_points(g, w, ctx->pkeys, ctx->pvals, ctx->stream);
         g.order = ctx->pvals[cur];
+        g.order_err = w.err;
     }
     GD_CUDA(ctx, launch_point(g, ctx->sms, ctx->stream));
     if (!dev_out)

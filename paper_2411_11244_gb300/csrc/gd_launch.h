@@ -9,6 +9,16 @@
 namespace gd {
 
 // ---- BVH build (gd_build.cu)
+constexpr int kSortPasses = 8;  // 64-bit keys, 8 bits a pass
+constexpr int kFlagTies = 14;
+
+struct SortWork {
+    unsigned long long* status;  // look-back table, 256 words a tile
+    unsigned* hist;              // digit counts, 256 a pass
+    unsigned* ticket;            // next tile of each pass
+    unsigned* err;               // a wait gave up
+};
+
 struct BuildBuffers {
     const float* verts;   // nv x 3, device
     const int32_t* tris;  // nt x 3, device
@@ -20,23 +30,30 @@ struct BuildBuffers {
     unsigned* order;      // nt, device: original index of each sorted triangle (kept for refits)
     int32_t* stris;       // nt x 3, device: the sorted triangles' vertex indices (written by the
                           // build, read by refits; may be nullptr for a build that keeps none)
-    unsigned* flags;      // device: [0] bad index, [1] non-finite vertex, [2..8] bounds scratch
+    unsigned* flags;      // device, 16 words: [0] bad index, [1] non-finite vertex, [2..8] bounds scratch,
+                          // [kFlagTies] more equal keys than the shortened sort can order
     unsigned long long* keys[2];  // nt each, device
     unsigned* vals[2];            // nt each, device
-    unsigned* hist;       // 256 * nblocks, device
+    SortWork sort;
 };
 
-size_t build_hist_words(long long nt);
-// stable LSD radix sort of n (key, value) pairs on the low key_bits bits of
-// the keys, 8 bits per pass, ping-ponging between keys[0|1] and vals[0|1]
-// (hist: build_hist_words(n) words); returns the index of the buffers that
-// hold the sorted pairs
-int radix_sort_pairs(unsigned long long* const keys[2], unsigned* const vals[2], long long n, int key_bits,
-                     unsigned* hist, cudaStream_t stream);
+// Stable LSD radix sort of n (key, value) pairs on the 8 passes key bits from
+// lo_bit up; the keys start in keys[0], their values are 0, 1, 2, ...; returns
+// the index of the buffers that hold the sorted pairs.  Before it, sort_clear,
+// then a kernel that adds the keys' digits to w.hist (256 words a pass).
+// scratch: sort_scratch_bytes(n) bytes, 8-byte aligned.  A bounded wait that gave
+// up sets *w.err (device), and the sorted buffers are then not written.
+size_t sort_scratch_bytes(long long n);
+SortWork sort_scratch(void* p, long long n);
+cudaError_t sort_clear(const SortWork& w, long long n, cudaStream_t stream);
+int radix_sort_pairs(const SortWork& w, unsigned long long* const keys[2], unsigned* const vals[2], long long n,
+                     int lo_bit, int passes, cudaStream_t stream);
 // checks indices and finiteness, and bounds the referenced vertices (flags)
 cudaError_t build_validate(const BuildBuffers& b, cudaStream_t stream);
-// the rest of the build; only after build_validate reported clean flags
-cudaError_t build_tree(const BuildBuffers& b, cudaStream_t stream);
+// the rest of the build; only after build_validate reported clean flags.  The
+// sort takes as many key bits as the triangle count calls for; flags[kFlagTies]
+// != 0 afterwards: too many triangles share those, build again with all_bits
+cudaError_t build_tree(const BuildBuffers& b, bool all_bits, cudaStream_t stream);
 // refit of a built tree after its vertices moved (verts, tris, L, order, tri,
 // box, flags): stored triangles and leaf boxes from the new vertices, then the
 // unions up to the root.  flags[1] != 0 afterwards: a referenced coordinate is
@@ -129,6 +146,7 @@ struct PointArgs {
     long long n;
     gd_point_result* out; // n results, device
     const unsigned* order;// order of work: the i-th point taken is order[i] (nullptr: point i)
+    const unsigned* order_err;  // device: != 0, order was not written (used with order)
     unsigned long long* ws;
     long long timeout_ns;
     unsigned epoch;       // differs from call to call
@@ -139,10 +157,9 @@ struct PointArgs {
     PointPart* parts;     // kPointMaxSlots + kPointMaxShares
 };
 
-// order the points along a Morton curve in the mesh's frame so that a warp's
-// walks visit the same nodes: keys[0], vals[0] in, sorted pairs in buffers
-// [returned index]; hist: build_hist_words(n) words
-int sort_points(const PointArgs& g, unsigned long long* const keys[2], unsigned* const vals[2], unsigned* hist,
+// order the points along a Morton curve in the mesh's frame so that nearby
+// points are walked at the same time: the indices end in vals[returned index]
+int sort_points(const PointArgs& g, const SortWork& w, unsigned long long* const keys[2], unsigned* const vals[2],
                 cudaStream_t stream);
 // sms: the device's SM count
 cudaError_t launch_point(PointArgs g, int sms, cudaStream_t stream);

@@ -694,6 +694,7 @@ __global__ void __launch_bounds__(kPointThreads, kPointCtas) k_point(const __gri
     __syncthreads();
     const unsigned lane = threadIdx.x & 31;
     PointWarp& W = s_w[threadIdx.x >> 5];
+    const unsigned* order = g.order && !*g.order_err ? g.order : nullptr;
     unsigned tests = 0, exact = 0;
     unsigned waiting = 0;  // candidates of finished points at the front of the list
     unsigned answered = 0; // points answered and not yet counted
@@ -729,7 +730,7 @@ __global__ void __launch_bounds__(kPointThreads, kPointCtas) k_point(const __gri
             }
             bool fin = true;
             if (lane < m) {
-                const unsigned i = g.order ? g.order[t0 + lane] : (unsigned)(t0 + lane);
+                const unsigned i = order ? order[t0 + lane] : (unsigned)(t0 + lane);
                 fin = isfinite(g.pts[3ull * i]) && isfinite(g.pts[3ull * i + 1]) && isfinite(g.pts[3ull * i + 2]);
                 W.pi[lane] = fin ? i : kNone;
                 if (fin) {
@@ -847,26 +848,39 @@ __device__ __forceinline__ unsigned long long spread10(unsigned v) {
 }
 
 // Morton key of each point in the mesh's frame, quantised in the root box
-// (points outside clamp to its faces: the key only orders the work)
-__global__ void k_point_keys(PointArgs g, unsigned long long* keys, unsigned* vals) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n) return;
-    const double* P = g.pts + 3 * i;
-    const double w0 = P[0] - g.x[3], w1 = P[1] - g.x[7], w2 = P[2] - g.x[11];
-    const double l[3] = {g.x[0] * w0 + g.x[4] * w1 + g.x[8] * w2, g.x[1] * w0 + g.x[5] * w1 + g.x[9] * w2,
-                         g.x[2] * w0 + g.x[6] * w1 + g.x[10] * w2};
-    unsigned long long key = 0;
+// (points outside clamp to its faces: the key only orders the work), and the
+// counts of its digits for the sort's passes
+constexpr int kKeyPasses = 4;  // 30 bits
+
+__global__ void __launch_bounds__(256) k_point_keys(const __grid_constant__ PointArgs g, unsigned long long* keys,
+                                                    unsigned* hist) {
+    __shared__ unsigned h[kKeyPasses][256];
+    for (int p = 0; p < kKeyPasses; ++p) h[p][threadIdx.x] = 0u;
+    __syncthreads();
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.n; i += (long long)gridDim.x * blockDim.x) {
+        const double* P = g.pts + 3 * i;
+        const double w0 = P[0] - g.x[3], w1 = P[1] - g.x[7], w2 = P[2] - g.x[11];
+        const double l[3] = {g.x[0] * w0 + g.x[4] * w1 + g.x[8] * w2, g.x[1] * w0 + g.x[5] * w1 + g.x[9] * w2,
+                             g.x[2] * w0 + g.x[6] * w1 + g.x[10] * w2};
+        unsigned long long key = 0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float lo = g.box[6 + k], hi = g.box[9 + k];
-        const float ext = hi - lo;
-        float f = ext > 0.f ? (float)((l[k] - lo) / ext) : 0.f;
-        f = f == f ? fminf(fmaxf(f, 0.f), 1.f) : 0.f;  // NaN (a non-finite point) to 0
-        const unsigned c = min(1023u, (unsigned)(f * 1024.f));
-        key |= spread10(c) << k;
+        for (int k = 0; k < 3; ++k) {
+            const float lo = g.box[6 + k], hi = g.box[9 + k];
+            const float ext = hi - lo;
+            float f = ext > 0.f ? (float)((l[k] - lo) / ext) : 0.f;
+            f = f == f ? fminf(fmaxf(f, 0.f), 1.f) : 0.f;  // NaN (a non-finite point) to 0
+            const unsigned c = min(1023u, (unsigned)(f * 1024.f));
+            key |= spread10(c) << k;
+        }
+        keys[i] = key;
+#pragma unroll
+        for (int p = 0; p < kKeyPasses; ++p) atomicAdd(&h[p][(unsigned)(key >> (8 * p)) & 255u], 1u);
     }
-    keys[i] = key;
-    vals[i] = (unsigned)i;
+    __syncthreads();
+    for (int p = 0; p < kKeyPasses; ++p) {
+        const unsigned n = h[p][threadIdx.x];
+        if (n) atomicAdd(hist + 256 * p + threadIdx.x, n);
+    }
 }
 
 __global__ void k_point_init(unsigned long long* ws) {
@@ -876,10 +890,11 @@ __global__ void k_point_init(unsigned long long* ws) {
 
 }  // namespace
 
-int sort_points(const PointArgs& g, unsigned long long* const keys[2], unsigned* const vals[2], unsigned* hist,
+int sort_points(const PointArgs& g, const SortWork& w, unsigned long long* const keys[2], unsigned* const vals[2],
                 cudaStream_t st) {
-    k_point_keys<<<(unsigned)((g.n + 255) / 256), 256, 0, st>>>(g, keys[0], vals[0]);
-    return radix_sort_pairs(keys, vals, g.n, 30, hist, st);
+    sort_clear(w, g.n, st);
+    k_point_keys<<<(unsigned)std::min(152ll * 8, (g.n + 255) / 256), 256, 0, st>>>(g, keys[0], w.hist);
+    return radix_sort_pairs(w, keys, vals, g.n, 0, kKeyPasses, st);
 }
 
 cudaError_t launch_point(PointArgs g, int sms, cudaStream_t st) {

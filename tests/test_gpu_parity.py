@@ -168,6 +168,64 @@ def _check_tree(boxes, order, v, t, L):
         assert np.array_equal(boxes[i][3:], np.maximum(l[3:], r[3:]))
 
 
+def _check_order_and_tree(G, h, v, t, bits=21):
+    boxes, order = G.gd_mesh_download(h)
+    assert np.array_equal(order, np.argsort(_morton_np(v, t, bits), kind="stable").astype(np.int32))
+    T, L = len(t), int(math.log2(len(t)))
+    vt = np.asarray(v, dtype=np.float32)[np.asarray(t)[order]]
+    first = (np.arange((1 << L) + 1, dtype=np.int64) * T) >> L
+    lo, hi = np.minimum.reduceat(vt.min(1), first[:-1]), np.maximum.reduceat(vt.max(1), first[:-1])
+    assert np.array_equal(boxes[1 << L:], np.concatenate([lo, hi], 1))
+    l, r = boxes[2:2 << L:2], boxes[3:2 << L:2]
+    assert np.array_equal(boxes[1:1 << L, :3], np.minimum(l[:, :3], r[:, :3]))
+    assert np.array_equal(boxes[1:1 << L, 3:], np.maximum(l[:, 3:], r[:, 3:]))
+
+
+@pytest.mark.parametrize("T", [7, 255, 256, 257, 511, 1023, 1024, 1025, 4097, 65536, (1 << 18) - 1, 1 << 18,
+                               (1 << 18) + 1, 300_001])
+def test_bvh_build_sort_sizes(G, ctx, T):
+    """Tile edges of both sort forms (1,024 and 4,096 keys, the change at
+    2^18), subtree edges of the leaf kernel."""
+    rng = np.random.default_rng(T)
+    v, t = _soup(rng, T, 1.0)
+    v[:, 2] *= 0.01
+    h = _mesh(G, ctx, (v, t))
+    try:
+        _check_order_and_tree(G, h, v, t)
+    finally:
+        G.gd_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("case", ["same", "run127", "run128", "run129", "cluster", "two_scales"])
+@pytest.mark.parametrize("bits", [21, 8, 1])
+def test_bvh_build_equal_keys(G, ctx, case, bits):
+    """Triangles that share the key bits the shortened sort looks at: runs
+    about as long as it orders itself (128), longer ones, and whole meshes
+    of them, which sort on all bits."""
+    rng = np.random.default_rng(7)
+    T = 5000
+    c = rng.uniform(-1, 1, (T, 3))
+    if case == "same":
+        c[:] = c[0]
+    elif case.startswith("run"):
+        n = int(case[3:])
+        c[100:100 + n] = c[100] + rng.uniform(0, 1e-5, (n, 3))
+    elif case == "cluster":
+        c[1:] = c[1] + rng.uniform(0, 1e-4, (T - 1, 3))
+    else:
+        c[: T // 2] *= 1e-3
+    c = rng.permutation(c)
+    v = (c[:, None, :] + rng.uniform(0, 1e-6, (T, 3, 3))).astype(np.float32).reshape(-1, 3)
+    t = np.arange(3 * T, dtype=np.int32).reshape(T, 3)
+    h = G.gd_mesh_create(ctx, v, t)
+    try:
+        for _ in range(2):
+            G.gd_bvh_build(h, bits, ctx=ctx)
+            _check_order_and_tree(G, h, v, t, bits)
+    finally:
+        G.gd_mesh_destroy(h)
+
+
 def test_bvh_build_rejects_bad_input(G, ctx):
     v = np.zeros((3, 3), np.float32)
     t = np.array([[0, 1, 3]], np.int32)
