@@ -411,14 +411,30 @@ __global__ void __launch_bounds__(256) k_order(const unsigned long long* keys, c
 
 constexpr int kTreeLevels = 8;  // tree levels one CTA reduces (2^8 = 256 nodes in, one out)
 
+// A run of shared memory to global memory by the bulk copy engine (one thread;
+// both addresses multiples of 16, and the size).  The threads that wrote the
+// run call bulk_ready before the barrier in front of it; the issuing thread
+// calls bulk_done before it leaves.
+__device__ __forceinline__ void bulk_ready() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
+                 "r"((unsigned)__cvta_generic_to_shared(src)), "r"(bytes)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_done() {
+    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
+}
+
 // Subtree union shared by the two tree kernels: on entry hb holds the 2^levels
 // boxes of the CTA's consecutive nodes of depth d (heap ids from first) at heap
 // positions 2^levels .. 2^(levels+1)-1, six floats each; every step makes node k
 // the union of its children 2k, 2k+1 (Section 4: tight children make a tight
-// parent).  The boxes of all levels (from row 0 up to row rows - 1) then go out
-// as runs of 8-byte words, a warp's words next to one another.  At the root
-// (depth 0) the root box goes to root_out[0..5] and max |coordinate| to *P_out,
-// when given.
+// parent).  The rows of boxes (from row 0 up to row rows - 1) then go out, each
+// a run of its own: 48 bytes times a whole number from an even node on, so the
+// copy engine takes all but the first.  At the root (depth 0) the root box goes
+// to root_out[0..5] and max |coordinate| to *P_out, when given.
 __device__ __forceinline__ void reduce_subtree(float* hb, float* box, long long first, int levels, int rows,
                                                float* root_out, float* P_out) {
     const int tid = threadIdx.x;
@@ -434,21 +450,19 @@ __device__ __forceinline__ void reduce_subtree(float* hb, float* box, long long 
             o[2] = make_float2(fmaxf(b.x, c.z), fmaxf(b.y, c.w));
         }
     }
+    bulk_ready();
     __syncthreads();
-    const float2* h2 = reinterpret_cast<const float2*>(hb);
-    float2* b2 = reinterpret_cast<float2*>(box);
     const long long root = first >> levels;
-    for (int i = 3 + tid; i < 3 * (1 << rows); i += blockDim.x) {
-        const int k = i / 3, rel = 31 - __clz(k);
-        b2[3 * ((root << rel) + (k - (1 << rel))) + (i - 3 * k)] = h2[i];
-    }
-    if (root == 1 && tid == 0) {
+    if (tid == 0) {
+        for (int r = 1; r < rows; ++r) bulk_store(box + 6 * (root << r), hb + (6 << r), 24u << r);
         float P = 0.f;
         for (int c = 0; c < 6; ++c) {
-            if (root_out) root_out[c] = hb[6 + c];
+            box[6 * root + c] = hb[6 + c];
+            if (root == 1 && root_out) root_out[c] = hb[6 + c];
             P = fmaxf(P, fabsf(hb[6 + c]));
         }
-        if (P_out) *P_out = P;
+        if (root == 1 && P_out) *P_out = P;
+        bulk_done();
     }
 }
 
@@ -463,19 +477,19 @@ __device__ __forceinline__ void reduce_subtree(float* hb, float* box, long long 
 // dependent ones.
 // bad != nullptr: a non-finite coordinate sets *bad (the refit's check; the
 // build validated the vertices before sorting).
-// Bound: the stores (48 bytes a triangle, 24 a node).  A thread per leaf that
-// stored its records and boxes itself wrote every 32-byte sector in two or
-// three pieces and filled the load/store queue: 7.5 M triangles took 228 us in
-// the build and 2 M 66 us in a refit; this form takes 188 and 46 (4.1 TB/s of
-// DRAM, the L1 busy 75 % of the time with the vertex gathers).
-__global__ void __launch_bounds__(1 << kTreeLevels)
+// Bound: the stores (48 bytes a triangle, 24 a node), which the copy engine
+// takes as runs.  A thread per leaf that stored its records and boxes itself
+// wrote every 32-byte sector in two or three pieces; one update of 7.5 M
+// triangles, copy and call included, took 204 us so, 212 with four CTAs an SM of
+// this form (64 registers), 196 with six.
+__global__ void __launch_bounds__(1 << kTreeLevels, 6)
     k_leaves(const float* verts, const int32_t* tris, long long nt, int L, const unsigned* order,
              const int32_t* stris_in, int32_t* stris_out, float4* tri, float* box, int levels, unsigned* bad,
              float* root_out, float* P_out) {
     constexpr int kMost = 2 << kTreeLevels;  // triangles of 2^kTreeLevels leaves
-    __shared__ float4 s_rec[3 * kMost];      // then the boxes, six floats a node
-    __shared__ int s_idx[3 * kMost];
-    static_assert(sizeof(s_rec) >= sizeof(float) * 6 * kMost, "the boxes take the records' place");
+    __shared__ float4 s_rec[3 * kMost];
+    __shared__ __align__(16) float hb[6 * kMost];  // the vertex indices, then the boxes
+    int* s_idx = reinterpret_cast<int*>(hb);
     const int tid = threadIdx.x;
     const long long l0 = (long long)blockIdx.x << levels;  // the CTA's first leaf
     const long long j0 = (long long)(((unsigned long long)l0 * (unsigned long long)nt) >> L);
@@ -520,10 +534,13 @@ __global__ void __launch_bounds__(1 << kTreeLevels)
             }
         }
     }
+    bulk_ready();
     if (__syncthreads_or(!finite) && bad && tid == 0) atomicOr(bad, 1u);
-    for (int i = tid; i < 3 * m; i += blockDim.x) tri[3 * j0 + i] = s_rec[i];
-    if (stris_out)
+    if (tid == 0) bulk_store(tri + 3 * j0, s_rec, 48u * (unsigned)m);
+    if (stris_out) {
         for (int i = tid; i < 3 * m; i += blockDim.x) stris_out[3 * j0 + i] = s_idx[i];
+        __syncthreads();
+    }
     float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
     {
         const long long l = l0 + tid;
@@ -540,8 +557,6 @@ __global__ void __launch_bounds__(1 << kTreeLevels)
             hi[2] = fmaxf(hi[2], fmaxf(p.z, fmaxf(q.y, z)));
         }
     }
-    __syncthreads();  // the records have been read
-    float* hb = reinterpret_cast<float*>(s_rec);
     float2* o = reinterpret_cast<float2*>(hb + 6 * ((1 << levels) + tid));
     o[0] = make_float2(lo[0], lo[1]);
     o[1] = make_float2(lo[2], hi[0]);
