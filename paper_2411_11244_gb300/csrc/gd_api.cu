@@ -42,7 +42,7 @@ struct gd_mesh {
     int32_t* d_stris = nullptr;   // vertex indices of each sorted triangle (leaf order), for refits
     MeshDev* d_desc = nullptr;
     MeshDev h_desc{};
-    unsigned* d_flags = nullptr;  // validation flags of gd_mesh_update
+    unsigned* d_flags = nullptr;  // flags of builds and updates (behind the descriptor)
     bool tree = false;            // box, tri and L hold a sorted tree (refit may run)
     bool built = false;           // ... and its boxes bound the current vertices
     float build_ms = 0.f;         // device time of the last build's kernels
@@ -52,6 +52,7 @@ struct gd_ctx {
     int device = 0;
     int sms = 0;
     cudaStream_t stream = nullptr;
+    cudaMemPool_t pool = nullptr;  // the meshes' buffers
     std::string err;
     gd_tunables tun{};
     // work buffers
@@ -94,10 +95,9 @@ struct gd_ctx {
     double* pts_dev = nullptr;               // staged host points and results
     gd_point_result* pres_dev = nullptr;
     long long cap_pts = 0;
-    unsigned long long* pkeys[2] = {nullptr, nullptr};  // Morton ordering of the points
-    unsigned* pvals[2] = {nullptr, nullptr};
-    void* psort = nullptr;
-    long long cap_psort = 0;
+    char* sort_mem = nullptr;    // keys, values and scratch of a sort (builds, points' order)
+    size_t cap_sort = 0;
+    cudaEvent_t build_ev[2] = {nullptr, nullptr};  // around a build's kernels
     unsigned long long last_point_tests = 0, last_point_exact = 0;  // counters of the last point call
     gd_stats last{};
     bool stats_pending = false;  // last run was device-resident: stats still on the device
@@ -124,6 +124,63 @@ gd_status cuda_fail(gd_ctx* ctx, cudaError_t e, const char* where) {
         cudaError_t e_ = (call);                                   \
         if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call); \
     } while (0)
+
+// Mesh buffers come from a pool of the context, which keeps up to kPoolKeep
+// bytes of what destroyed meshes leave (cudaMalloc and cudaFree map and unmap
+// whatever exceeds 1 MB on every call: 0.1 ms and more each).  The memory is
+// allocated and freed in the order of the context's stream; the calls that make a
+// mesh synchronise that stream before they return, and gd_mesh_destroy the
+// device before it frees.
+constexpr unsigned long long kPoolKeep = 256ull << 20;
+
+template <class T>
+cudaError_t mesh_alloc(gd_ctx* c, T** p, size_t bytes) {
+    if (*p) return cudaSuccess;  // sizes follow from the mesh: a rebuild keeps its buffers
+    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, c->pool, c->stream);
+}
+
+template <class T>
+void mesh_free(gd_ctx* c, T* p) {
+    if (p) cudaFreeAsync(p, c->stream);
+}
+
+// Buffers of a sort of n keys.  One allocation a context, reused by its builds
+// and point queries, which all run on its stream; above kSortKeep it is given
+// back at the end of the call (drop_sort), so that one huge mesh does not hold it.
+constexpr size_t kSortKeep = 1ull << 30;
+
+struct SortBuffers {
+    unsigned long long* keys[2];
+    unsigned* vals[2];
+    SortWork work;
+};
+
+cudaError_t sort_buffers(gd_ctx* c, long long n, SortBuffers* b) {
+    const size_t k = (sizeof(unsigned long long) * (size_t)n + 255) / 256 * 256;
+    const size_t v = (sizeof(unsigned) * (size_t)n + 255) / 256 * 256;
+    const size_t need = 2 * (k + v) + sort_scratch_bytes(n);
+    if (need > c->cap_sort) {
+        cudaFree(c->sort_mem);
+        c->sort_mem = nullptr;
+        c->cap_sort = 0;
+        const cudaError_t e = cudaMalloc(&c->sort_mem, need);
+        if (e != cudaSuccess) return e;
+        c->cap_sort = need;
+    }
+    for (int i = 0; i < 2; ++i) {
+        b->keys[i] = reinterpret_cast<unsigned long long*>(c->sort_mem + i * k);
+        b->vals[i] = reinterpret_cast<unsigned*>(c->sort_mem + 2 * k + i * v);
+    }
+    b->work = sort_scratch(c->sort_mem + 2 * (k + v), n);
+    return cudaSuccess;
+}
+
+void drop_sort(gd_ctx* c) {
+    if (c->cap_sort <= kSortKeep) return;
+    cudaFree(c->sort_mem);
+    c->sort_mem = nullptr;
+    c->cap_sort = 0;
+}
 
 bool xform_ok(const double* x, std::string* why) {
     for (int i = 0; i < 12; ++i)
@@ -546,6 +603,18 @@ GD_API gd_status gd_ctx_create(int device, gd_ctx** out) {
         delete c;
         return GD_ERR_CUDA;
     }
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        if (c->pool) cudaMemPoolDestroy(c->pool);
+        cudaStreamDestroy(c->stream);
+        delete c;
+        return GD_ERR_CUDA;
+    }
     c->tun.work_target = 1ll << 17;
     c->tun.k_max = 6;
     c->tun.blocks_per_sm = 0;
@@ -577,8 +646,11 @@ GD_API void gd_ctx_destroy(gd_ctx* c) {
     cudaFree(c->ftree);
     cudaFree(c->naive_ws);
     cudaFree(c->point_ws); cudaFree(c->point_share); cudaFree(c->pts_dev); cudaFree(c->pres_dev);
-    cudaFree(c->pkeys[0]); cudaFree(c->pkeys[1]); cudaFree(c->pvals[0]); cudaFree(c->pvals[1]);
-    cudaFree(c->psort);
+    cudaFree(c->sort_mem);
+    for (cudaEvent_t e : c->build_ev)
+        if (e) cudaEventDestroy(e);
+    cudaStreamSynchronize(c->stream);
+    cudaMemPoolDestroy(c->pool);
     cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -717,8 +789,8 @@ GD_API gd_status gd_mesh_create(gd_ctx* ctx, const float* verts, int64_t nv, con
     m->ctx = ctx;
     m->nv = nv;
     m->nt = nt;
-    cudaError_t e = cudaMalloc(&m->d_verts, sizeof(float) * 3 * nv);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_tris, sizeof(int32_t) * 3 * nt);
+    cudaError_t e = mesh_alloc(ctx, &m->d_verts, sizeof(float) * 3 * nv);
+    if (e == cudaSuccess) e = mesh_alloc(ctx, &m->d_tris, sizeof(int32_t) * 3 * nt);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->d_verts, verts, sizeof(float) * 3 * nv, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->d_tris, tris, sizeof(int32_t) * 3 * nt, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -729,6 +801,39 @@ GD_API gd_status gd_mesh_create(gd_ctx* ctx, const float* verts, int64_t nv, con
     *out = m;
     return GD_OK;
 }
+
+namespace {
+cudaError_t tree_buffers(gd_mesh* m, int L) {
+    gd_ctx* c = m->ctx;
+    const size_t nt = (size_t)m->nt;
+    cudaError_t e = mesh_alloc(c, &m->d_box, sizeof(float) * 6 * (2ull << L));
+    if (e == cudaSuccess) e = mesh_alloc(c, &m->d_tri, sizeof(float4) * 3 * nt);
+    if (e == cudaSuccess) e = mesh_alloc(c, &m->d_order, sizeof(unsigned) * nt);
+    if (e == cudaSuccess) e = mesh_alloc(c, &m->d_stris, sizeof(int32_t) * 3 * nt);
+    // (the descriptors of all meshes, which every query reads first, on one small page)
+    if (e == cudaSuccess && !m->d_desc) {
+        e = cudaMalloc(&m->d_desc, 128 + 16 * sizeof(unsigned));
+        if (e == cudaSuccess) m->d_flags = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(m->d_desc) + 128);
+    }
+    static_assert(sizeof(MeshDev) <= 128, "the flags follow the descriptor");
+    return e;
+}
+
+float* desc_P(const gd_mesh* m) {
+    return reinterpret_cast<float*>(reinterpret_cast<char*>(m->d_desc) + offsetof(MeshDev, P));
+}
+
+// max |coordinate| of the root box in flags[8..13]
+float root_P(const unsigned* flags) {
+    float P = 0.f;
+    for (int i = 0; i < 6; ++i) {
+        float x;
+        std::memcpy(&x, &flags[8 + i], sizeof(float));
+        P = std::max(P, std::fabs(x));
+    }
+    return P;
+}
+}  // namespace
 
 GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     if (!m) return GD_ERR_INVALID_ARG;
@@ -741,90 +846,55 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     }
     int L = 0;
     while ((2ll << L) <= m->nt) ++L;
-    cudaFree(m->d_box); cudaFree(m->d_tri); cudaFree(m->d_order); cudaFree(m->d_stris);
-    m->d_box = nullptr; m->d_tri = nullptr; m->d_order = nullptr; m->d_stris = nullptr;
+    // a tree that work on any stream may still read is only overwritten once that is done
+    if (m->d_desc) GD_CUDA(ctx, cudaDeviceSynchronize());
     m->built = false;
     m->tree = false;
     BuildBuffers b{};
+    SortBuffers sb{};
+    cudaError_t e = tree_buffers(m, L);
+    if (e == cudaSuccess) e = sort_buffers(ctx, m->nt, &sb);
+    for (cudaEvent_t& x : ctx->build_ev)
+        if (e == cudaSuccess && !x) e = cudaEventCreate(&x);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "gd_bvh_build alloc");
+    struct Drop {
+        gd_ctx* c;
+        ~Drop() { drop_sort(c); }
+    } drop{ctx};
     b.verts = m->d_verts; b.tris = m->d_tris; b.nv = m->nv; b.nt = m->nt; b.L = L; b.morton_bits = bits;
-    std::vector<void*> tmp;
-    auto cleanup = [&]() { for (void* p : tmp) cudaFree(p); };
-#define GD_ALLOC(ptr, bytes)                                                 \
-    do {                                                                     \
-        cudaError_t e_ = cudaMalloc((void**)&(ptr), (bytes));                \
-        if (e_ != cudaSuccess) { cleanup(); return cuda_fail(ctx, e_, "gd_bvh_build alloc"); } \
-        tmp.push_back((void*)(ptr));                                         \
-    } while (0)
-    GD_ALLOC(b.flags, 64 * sizeof(unsigned));
-    GD_ALLOC(b.keys[0], sizeof(unsigned long long) * m->nt);
-    GD_ALLOC(b.keys[1], sizeof(unsigned long long) * m->nt);
-    GD_ALLOC(b.vals[0], sizeof(unsigned) * m->nt);
-    GD_ALLOC(b.vals[1], sizeof(unsigned) * m->nt);
-    void* sort_mem = nullptr;
-    GD_ALLOC(sort_mem, sort_scratch_bytes(m->nt));
-    b.sort = sort_scratch(sort_mem, m->nt);
-#undef GD_ALLOC
-    cudaError_t e = cudaMalloc(&m->d_box, sizeof(float) * 6 * (2ull << L));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_tri, sizeof(float4) * 3 * m->nt);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_order, sizeof(unsigned) * m->nt);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_stris, sizeof(int32_t) * 3 * m->nt);
-    if (e != cudaSuccess) { cleanup(); return cuda_fail(ctx, e, "gd_bvh_build alloc"); }
-    b.box = m->d_box;
-    b.tri = m->d_tri;
-    b.order = m->d_order;
-    b.stris = m->d_stris;
-    unsigned flags[8] = {0};
-    // device time of the build's kernels: events around the validation and
-    // around the tree build (not the allocations and the flag read-back)
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    for (cudaEvent_t& x : ev) cudaEventCreate(&x);
-    auto drop_events = [&]() { for (cudaEvent_t& x : ev) if (x) cudaEventDestroy(x); };
-    cudaEventRecord(ev[0], ctx->stream);
-    e = build_validate(b, ctx->stream);
-    cudaEventRecord(ev[1], ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(flags, b.flags, sizeof(flags), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) { drop_events(); cleanup(); return cuda_fail(ctx, e, "gd_bvh_build validate"); }
-    if (flags[0]) { drop_events(); cleanup(); return fail(ctx, GD_ERR_INVALID_ARG, "triangle index out of range"); }
-    if (flags[1]) { drop_events(); cleanup(); return fail(ctx, GD_ERR_INVALID_ARG, "non-finite vertex coordinate"); }
-    cudaEventRecord(ev[2], ctx->stream);
-    float root[6];
-    unsigned ties = 0, sort_err = 0;
-    for (int all_bits = 0; all_bits < 2 && e == cudaSuccess; ++all_bits) {
-        e = build_tree(b, all_bits != 0, ctx->stream);
-        cudaEventRecord(ev[3], ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(root, m->d_box + 6, sizeof(root), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&ties, b.flags + kFlagTies, sizeof(ties), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&sort_err, b.sort.err, sizeof(sort_err), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (!ties) break;
+    b.box = m->d_box; b.tri = m->d_tri; b.order = m->d_order; b.stris = m->d_stris; b.flags = m->d_flags;
+    for (int i = 0; i < 2; ++i) {
+        b.keys[i] = sb.keys[i];
+        b.vals[i] = sb.vals[i];
     }
-    cleanup();
-    if (e == cudaSuccess && sort_err) {
-        drop_events();
-        return fail(ctx, GD_ERR_TIMEOUT, "a device-side wait of the build's sort timed out");
-    }
-    if (e == cudaSuccess) {
-        float t0 = 0.f, t1 = 0.f;
-        cudaEventElapsedTime(&t0, ev[0], ev[1]);
-        cudaEventElapsedTime(&t1, ev[2], ev[3]);
-        m->build_ms = t0 + t1;
-    }
-    drop_events();
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "gd_bvh_build");
-    float P = 0.f;
-    for (int i = 0; i < 6; ++i) P = std::max(P, std::fabs(root[i]));
-    m->L = L;
+    b.sort = sb.work;
     m->h_desc.box = m->d_box;
     m->h_desc.tri = m->d_tri;
     m->h_desc.T = m->nt;
     m->h_desc.L = L;
-    m->h_desc.P = P;
-    if (!m->d_desc) GD_CUDA(ctx, cudaMalloc(&m->d_desc, sizeof(MeshDev)));
+    m->h_desc.P = 0.f;  // (the root's kernel writes the device's)
     GD_CUDA(ctx, cudaMemcpyAsync(m->d_desc, &m->h_desc, sizeof(MeshDev), cudaMemcpyHostToDevice, ctx->stream));
-    GD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    // device time of the build's kernels: events around them, on the stream they run on
+    unsigned flags[16];
+    for (int all_bits = 0; all_bits < 2; ++all_bits) {
+        if (!all_bits) {
+            cudaEventRecord(ctx->build_ev[0], ctx->stream);
+            e = build_validate(b, ctx->stream);
+        }
+        if (e == cudaSuccess) e = build_tree(b, all_bits != 0, desc_P(m), ctx->stream);
+        cudaEventRecord(ctx->build_ev[1], ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(flags, b.flags, sizeof(flags), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "gd_bvh_build");
+        if (flags[0]) return fail(ctx, GD_ERR_INVALID_ARG, "triangle index out of range");
+        if (flags[1]) return fail(ctx, GD_ERR_INVALID_ARG, "non-finite vertex coordinate");
+        if (flags[kFlagSort]) return fail(ctx, GD_ERR_TIMEOUT, "a device-side wait of the build's sort timed out");
+        if (!flags[kFlagTies]) break;
+    }
+    m->build_ms = 0.f;
+    cudaEventElapsedTime(&m->build_ms, ctx->build_ev[0], ctx->build_ev[1]);
+    m->h_desc.P = root_P(flags);
+    m->L = L;
     m->built = true;
     m->tree = true;
     return GD_OK;
@@ -838,38 +908,34 @@ GD_API gd_status gd_mesh_update(gd_mesh* m, const float* verts, int64_t nv) {
     if (!m->tree) return fail(ctx, GD_ERR_NOT_BUILT, "BVH not built (call gd_bvh_build)");
     cudaSetDevice(ctx->device);
     m->built = false;
-    if (!m->d_flags) GD_CUDA(ctx, cudaMalloc(&m->d_flags, 64 * sizeof(unsigned)));
     // host or device source: with unified addressing the copy kind follows the pointer
     GD_CUDA(ctx, cudaMemcpyAsync(m->d_verts, verts, sizeof(float) * 3 * nv, cudaMemcpyDefault, ctx->stream));
     BuildBuffers b{};
     b.verts = m->d_verts; b.tris = m->d_tris; b.nv = m->nv; b.nt = m->nt; b.L = m->L;
     b.box = m->d_box; b.tri = m->d_tri; b.order = m->d_order; b.stris = m->d_stris; b.flags = m->d_flags;
     // the refit writes max |coordinate| straight into the device descriptor
-    float* P_dev = reinterpret_cast<float*>(reinterpret_cast<char*>(m->d_desc) + offsetof(MeshDev, P));
-    GD_CUDA(ctx, build_refit(b, P_dev, ctx->stream));
+    GD_CUDA(ctx, build_refit(b, desc_P(m), ctx->stream));
     unsigned flags[14];
     GD_CUDA(ctx, cudaMemcpyAsync(flags, b.flags, sizeof(flags), cudaMemcpyDeviceToHost, ctx->stream));
     GD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (flags[1]) return fail(ctx, GD_ERR_INVALID_ARG, "non-finite vertex coordinate (mesh left unbuilt)");
-    float P = 0.f;
-    for (int i = 0; i < 6; ++i) {
-        float x;
-        std::memcpy(&x, &flags[8 + i], sizeof(float));
-        P = std::max(P, std::fabs(x));
-    }
-    m->h_desc.P = P;
+    m->h_desc.P = root_P(flags);
     m->built = true;
     return GD_OK;
 }
 
 GD_API void gd_mesh_destroy(gd_mesh* m) {
     if (!m) return;
-    if (m->ctx) {
-        cudaSetDevice(m->ctx->device);
-        cudaStreamSynchronize(m->ctx->stream);
-    }
-    cudaFree(m->d_verts); cudaFree(m->d_tris); cudaFree(m->d_box); cudaFree(m->d_tri); cudaFree(m->d_desc);
-    cudaFree(m->d_order); cudaFree(m->d_stris); cudaFree(m->d_flags);
+    gd_ctx* c = m->ctx;
+    cudaSetDevice(c->device);
+    cudaDeviceSynchronize();  // queries on any stream
+    mesh_free(c, m->d_verts);
+    mesh_free(c, m->d_tris);
+    mesh_free(c, m->d_box);
+    mesh_free(c, m->d_tri);
+    mesh_free(c, m->d_order);
+    mesh_free(c, m->d_stris);
+    cudaFree(m->d_desc);
     delete m;
 }
 
@@ -962,25 +1028,11 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
     // enough points to fill the GPU: walk them in Morton order (warps of
     // nearby points visit the same nodes)
     if (n >= kPointSortMin) {
-        if (n > ctx->cap_psort) {
-            for (int k = 0; k < 2; ++k) {
-                cudaFree(ctx->pkeys[k]); cudaFree(ctx->pvals[k]);
-                ctx->pkeys[k] = nullptr; ctx->pvals[k] = nullptr;
-            }
-            cudaFree(ctx->psort);
-            ctx->psort = nullptr;
-            ctx->cap_psort = 0;
-            for (int k = 0; k < 2; ++k) {
-                GD_CUDA(ctx, cudaMalloc(&ctx->pkeys[k], sizeof(unsigned long long) * n));
-                GD_CUDA(ctx, cudaMalloc(&ctx->pvals[k], sizeof(unsigned) * n));
-            }
-            GD_CUDA(ctx, cudaMalloc(&ctx->psort, std::max(sort_scratch_bytes(n), sort_scratch_bytes(1ll << 18))));
-            ctx->cap_psort = n;
-        }
-        const SortWork w = sort_scratch(ctx->psort, n);
-        const int cur = sort_points(g, w, ctx->pkeys, ctx->pvals, ctx->stream);
-        g.order = ctx->pvals[cur];
-        g.order_err = w.err;
+        SortBuffers sb{};
+        GD_CUDA(ctx, sort_buffers(ctx, n, &sb));
+        const int cur = sort_points(g, sb.work, sb.keys, sb.vals, ctx->stream);
+        g.order = sb.vals[cur];
+        g.order_err = sb.work.err;
     }
     GD_CUDA(ctx, launch_point(g, ctx->sms, ctx->stream));
     if (!dev_out)
@@ -988,6 +1040,7 @@ GD_API gd_status gd_point_distance(gd_ctx* ctx, const gd_mesh* M, const double x
     unsigned long long w[kPointWords];
     GD_CUDA(ctx, cudaMemcpyAsync(w, ctx->point_ws, sizeof(w), cudaMemcpyDeviceToHost, ctx->stream));
     GD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    drop_sort(ctx);
     ctx->last_point_tests = w[kPointTests];
     ctx->last_point_exact = w[kPointExact];
     if (w[kPointTimeout] || w[kPointAnswered] < (unsigned long long)n) return fail(ctx, GD_ERR_TIMEOUT, "a point query passed the timeout");

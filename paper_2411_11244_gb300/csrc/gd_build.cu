@@ -43,7 +43,8 @@ __device__ __forceinline__ void load_vertex(const float* verts, unsigned v, floa
     x[2] = p[2];
 }
 
-// flags: [0] bad index, [1] non-finite vertex, [2..4] ordered min, [5..7] ordered max, [kFlagTies]
+// flags: [0] bad index, [1] non-finite vertex, [2..4] ordered min, [5..7] ordered max,
+// [8..13] root box, [kFlagTies], [kFlagSort]
 __global__ void k_init_flags(unsigned* flags) {
     if (threadIdx.x < 16) flags[threadIdx.x] = (threadIdx.x >= 2 && threadIdx.x < 5) ? 0xffffffffu : 0u;
 }
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(512) k_morton(const float* verts, const int32_
     // one scale for all three axes (cubic cells): per-axis scales would make
     // the cells of flat or thin meshes into slabs whose boxes are far from
     // the surface they bound
+    const bool bad = flags[0] != 0u;  // an index out of range: the build fails, nothing is read through it
     float lo[3], ext[3], e = 0.f;
     for (int c = 0; c < 3; ++c) {
         lo[c] = unordered(flags[2 + c]);
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(512) k_morton(const float* verts, const int32_
             unsigned q[3];
             float v[9];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) load_vertex(verts, (unsigned)tris[3 * t + k], v + 3 * k);
+            for (int k = 0; k < 3; ++k) load_vertex(verts, bad ? 0u : (unsigned)tris[3 * t + k], v + 3 * k);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 // explicit round-to-nearest steps (no contraction), so that the
@@ -388,6 +390,7 @@ __global__ void __launch_bounds__(256) k_order(const unsigned long long* keys, c
         const long long i = base + k;
         if (i >= n) return;
         if (failed) {
+            if (i == 0) flags[kFlagSort] = 1u;
             order[i] = (unsigned)i;
             continue;
         }
@@ -476,7 +479,8 @@ __device__ __forceinline__ void reduce_subtree(float* hb, float* box, long long 
 // there, contiguously, so its vertex gathers wait on one load instead of two
 // dependent ones.
 // bad != nullptr: a non-finite coordinate sets *bad (the refit's check; the
-// build validated the vertices before sorting).
+// build's validation has made its own).  skip != nullptr and *skip != 0: the
+// build has met an index out of range and nothing is read through it.
 // Bound: the stores (48 bytes a triangle, 24 a node), which the copy engine
 // takes as runs.  A thread per leaf that stored its records and boxes itself
 // wrote every 32-byte sector in two or three pieces; one update of 7.5 M
@@ -485,11 +489,12 @@ __device__ __forceinline__ void reduce_subtree(float* hb, float* box, long long 
 __global__ void __launch_bounds__(1 << kTreeLevels, 6)
     k_leaves(const float* verts, const int32_t* tris, long long nt, int L, const unsigned* order,
              const int32_t* stris_in, int32_t* stris_out, float4* tri, float* box, int levels, unsigned* bad,
-             float* root_out, float* P_out) {
+             const unsigned* skip, float* root_out, float* P_out) {
     constexpr int kMost = 2 << kTreeLevels;  // triangles of 2^kTreeLevels leaves
     __shared__ float4 s_rec[3 * kMost];
     __shared__ __align__(16) float hb[6 * kMost];  // the vertex indices, then the boxes
     int* s_idx = reinterpret_cast<int*>(hb);
+    if (skip && *skip) return;
     const int tid = threadIdx.x;
     const long long l0 = (long long)blockIdx.x << levels;  // the CTA's first leaf
     const long long j0 = (long long)(((unsigned long long)l0 * (unsigned long long)nt) >> L);
@@ -577,11 +582,11 @@ __global__ void __launch_bounds__(1 << kTreeLevels)
 // all boxes from the sorted order: leaves plus the lowest levels, then one
 // launch per further kTreeLevels levels (three launches for 2^22 leaves)
 void tree_boxes(const float* verts, const int32_t* tris, long long nt, int L, const unsigned* order,
-                const int32_t* stris_in, int32_t* stris_out, float4* tri, float* box, unsigned* bad, float* root_out,
-                float* P_out, cudaStream_t st) {
+                const int32_t* stris_in, int32_t* stris_out, float4* tri, float* box, unsigned* bad,
+                const unsigned* skip, float* root_out, float* P_out, cudaStream_t st) {
     int lv = L < kTreeLevels ? L : kTreeLevels;
     k_leaves<<<(unsigned)(1ll << (L - lv)), 1u << lv, 0, st>>>(verts, tris, nt, L, order, stris_in, stris_out, tri, box,
-                                                                 lv, bad, root_out, P_out);
+                                                                 lv, bad, skip, root_out, P_out);
     for (int d = L - lv; d > 0; d -= lv) {
         lv = d < kTreeLevels ? d : kTreeLevels;
         k_reduce_up<<<(unsigned)(1ll << (d - lv)), 1u << lv, 0, st>>>(box, d, lv, root_out, P_out);
@@ -650,7 +655,7 @@ int build_passes(long long nt, int morton_bits) {
     return std::min(all, std::max(2, (3 * (lg + 1) / 2 + 6) / 8));
 }
 
-cudaError_t build_tree(const BuildBuffers& b, bool all_bits, cudaStream_t st) {
+cudaError_t build_tree(const BuildBuffers& b, bool all_bits, float* P_out, cudaStream_t st) {
     const int bits = 3 * b.morton_bits, all = (bits + 7) / 8;
     const int passes = all_bits ? all : build_passes(b.nt, b.morton_bits);
     const int lo = passes == all ? 0 : bits - 8 * passes;
@@ -661,7 +666,8 @@ cudaError_t build_tree(const BuildBuffers& b, bool all_bits, cudaStream_t st) {
     const int cur = radix_sort_pairs(b.sort, b.keys, b.vals, b.nt, lo, passes, st);
     k_order<<<(unsigned)((b.nt + kOrderTile - 1) / kOrderTile), 256, 0, st>>>(b.keys[cur], b.vals[cur], b.nt, lo, b.sort.err, b.order,
                                                              b.flags);
-    tree_boxes(b.verts, b.tris, b.nt, b.L, b.order, nullptr, b.stris, b.tri, b.box, nullptr, nullptr, nullptr, st);
+    tree_boxes(b.verts, b.tris, b.nt, b.L, b.order, nullptr, b.stris, b.tri, b.box, nullptr, b.flags,
+               reinterpret_cast<float*>(b.flags + 8), P_out, st);
     return cudaGetLastError();
 }
 
@@ -669,7 +675,7 @@ cudaError_t build_refit(const BuildBuffers& b, float* P_out, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(b.flags, 0, 16 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     tree_boxes(b.verts, b.tris, b.nt, b.L, b.order, b.stris, nullptr, b.tri, b.box, b.flags + 1,
-               reinterpret_cast<float*>(b.flags + 8), P_out, st);
+               nullptr, reinterpret_cast<float*>(b.flags + 8), P_out, st);
     return cudaGetLastError();
 }
 

@@ -10,7 +10,7 @@ namespace gd {
 
 // ---- BVH build (gd_build.cu)
 constexpr int kSortPasses = 8;  // 64-bit keys, 8 bits a pass
-constexpr int kFlagTies = 14;
+constexpr int kFlagTies = 14, kFlagSort = 15;
 
 struct SortWork {
     unsigned long long* status;  // look-back table, 256 words a tile
@@ -30,8 +30,9 @@ struct BuildBuffers {
     unsigned* order;      // nt, device: original index of each sorted triangle (kept for refits)
     int32_t* stris;       // nt x 3, device: the sorted triangles' vertex indices (written by the
                           // build, read by refits; may be nullptr for a build that keeps none)
-    unsigned* flags;      // device, 16 words: [0] bad index, [1] non-finite vertex, [2..8] bounds scratch,
-                          // [kFlagTies] more equal keys than the shortened sort can order
+    unsigned* flags;      // device, 16 words: [0] bad index, [1] non-finite vertex, [2..7] bounds of the
+                          // vertices, [8..13] the root box, [kFlagTies] more equal keys than the shortened
+                          // sort can order, [kFlagSort] a wait of the sort gave up
     unsigned long long* keys[2];  // nt each, device
     unsigned* vals[2];            // nt each, device
     SortWork sort;
@@ -50,10 +51,11 @@ int radix_sort_pairs(const SortWork& w, unsigned long long* const keys[2], unsig
                      int lo_bit, int passes, cudaStream_t stream);
 // checks indices and finiteness, and bounds the referenced vertices (flags)
 cudaError_t build_validate(const BuildBuffers& b, cudaStream_t stream);
-// the rest of the build; only after build_validate reported clean flags.  The
-// sort takes as many key bits as the triangle count calls for; flags[kFlagTies]
-// != 0 afterwards: too many triangles share those, build again with all_bits
-cudaError_t build_tree(const BuildBuffers& b, bool all_bits, cudaStream_t stream);
+// the rest of the build, after build_validate (its kernels read nothing through
+// an index that is out of range).  The sort takes as many key bits as the
+// triangle count calls for; flags[kFlagTies] != 0 afterwards: too many triangles
+// share those, build again with all_bits.  *P_out: max |coordinate| of the root box
+cudaError_t build_tree(const BuildBuffers& b, bool all_bits, float* P_out, cudaStream_t stream);
 // refit of a built tree after its vertices moved (verts, tris, L, order, tri,
 // box, flags): stored triangles and leaf boxes from the new vertices, then the
 // unions up to the root.  flags[1] != 0 afterwards: a referenced coordinate is
