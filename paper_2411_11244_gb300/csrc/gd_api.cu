@@ -30,6 +30,17 @@ struct Mailbox {
 };
 constexpr size_t kResultBytes = offsetof(Mailbox, stats);
 
+// What a single query's CTA 0 reads and writes all the time, on one page: a
+// context tries kPages of them and takes the one nearest to that CTA (see
+// k_near_page).
+constexpr size_t kPageBytes = 4096;
+constexpr int kPages = 16;
+struct SinglePage {
+    Mailbox mb;
+    QState q;
+};
+static_assert(sizeof(SinglePage) <= kPageBytes, "one page");
+
 struct gd_mesh {
     gd_ctx* ctx = nullptr;
     long long nv = 0, nt = 0;
@@ -63,7 +74,9 @@ struct gd_ctx {
     double* cand_d = nullptr;
     double* cand_pts = nullptr;
     long long cap_front = 0, cap_leaf = 0, cap_cand = 0;
+    char* pages = nullptr;       // kPages pages, of which one holds mb_dev and qs_one
     Mailbox* mb_dev = nullptr;   // single-query results, stats and counters
+    QState* qs_one = nullptr;    // a single query's state
     Mailbox* mb_host = nullptr;  // pinned mirror
     HostDone* hd = nullptr;      // pinned result records, written by the kernel: [0] for the
                                  // synchronous calls, [1..kPipe] for the server's pipelined launches
@@ -259,11 +272,23 @@ gd_status alloc_queues(gd_ctx* c) {
 
 gd_status ensure_ws(gd_ctx* c, long long nq) {
     if (!c->mb_dev) {
-        GD_CUDA(c, cudaMalloc(&c->mb_dev, sizeof(Mailbox)));
-        GD_CUDA(c, cudaMemset(c->mb_dev, 0, sizeof(Mailbox)));
-        GD_CUDA(c, cudaMallocHost(&c->mb_host, sizeof(Mailbox)));
-        GD_CUDA(c, cudaMallocHost(&c->hd, sizeof(HostDone) * (1 + kPipe)));
+        if (!c->pages) GD_CUDA(c, cudaMalloc(&c->pages, kPageBytes * (kPages + 1)));
+        if (!c->mb_host) GD_CUDA(c, cudaMallocHost(&c->mb_host, sizeof(Mailbox)));
+        if (!c->hd) GD_CUDA(c, cudaMallocHost(&c->hd, sizeof(HostDone) * (1 + kPipe)));
         std::memset(c->hd, 0, sizeof(HostDone) * (1 + kPipe));
+        // page-aligned (the allocation is aligned to 256 bytes only by contract)
+        char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(c->pages) + kPageBytes - 1) / kPageBytes * kPageBytes);
+        unsigned* found = reinterpret_cast<unsigned*>(base + kPageBytes - 64);  // (beyond a SinglePage)
+        static_assert(sizeof(SinglePage) <= kPageBytes - 64, "room for the result");
+        unsigned page = 0;
+        GD_CUDA(c, cudaMemsetAsync(base, 0, kPageBytes * kPages, c->stream));
+        GD_CUDA(c, launch_near_page(reinterpret_cast<unsigned*>(base), kPages, kPageBytes / sizeof(unsigned), found,
+                                    2 * c->sms, c->stream));
+        GD_CUDA(c, cudaMemcpyAsync(&page, found, sizeof(page), cudaMemcpyDeviceToHost, c->stream));
+        GD_CUDA(c, cudaStreamSynchronize(c->stream));
+        SinglePage* sp = reinterpret_cast<SinglePage*>(base + kPageBytes * std::min(page, (unsigned)kPages - 1u));
+        c->qs_one = &sp->q;
+        c->mb_dev = &sp->mb;
     }
     if (!c->ready) {
         c->cap_front = std::min<long long>(c->tun.front_capacity, 0xffffffffll);
@@ -453,6 +478,7 @@ gd_status run_single(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B, int kind, 
         std::memcpy(a.xa_val, xa, sizeof(a.xa_val));
         std::memcpy(a.xb_val, xb, sizeof(a.xb_val));
         fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
+        a.qs = ctx->qs_one;
         a.slot_of = ctx->slot_of;
         a.n_slot_of = (unsigned long long)tab;
         a.out = &ctx->mb_dev->out;
@@ -637,7 +663,7 @@ GD_API void gd_ctx_destroy(gd_ctx* c) {
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     free_ws(c);
-    cudaFree(c->mb_dev);
+    cudaFree(c->pages);
     cudaFreeHost(c->mb_host);
     cudaFreeHost(c->hd);
     cudaFree(c->qs); cudaFree(c->qin_dev); cudaFree(c->out_dev); cudaFree(c->done_dev);
@@ -1134,6 +1160,7 @@ GD_API gd_status gd_query_device(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B
     fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
     a.slot_of = ctx->slot_of;
     a.n_slot_of = (unsigned long long)tab;
+    a.qs = ctx->qs_one;
     a.out = d_out;
     s = full_refit_tree(ctx, B, a);
     if (s != GD_OK) return s;
@@ -1175,6 +1202,7 @@ gd_status graph_build(gd_graph* g) {
     fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
     a.slot_of = ctx->slot_of;
     a.n_slot_of = (unsigned long long)tab;
+    a.qs = ctx->qs_one;
     a.out = g->d_out;
     s = full_refit_tree(ctx, g->B, a);
     if (s != GD_OK) return s;
@@ -1354,6 +1382,7 @@ gd_status serve_single_launch(gd_ctx* ctx, const gd_query& q, int slot, unsigned
     fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
     a.slot_of = ctx->slot_of;
     a.n_slot_of = (unsigned long long)tab;
+    a.qs = ctx->qs_one;
     a.out = &ctx->mb_dev->out;
     s = full_refit_tree(ctx, B, a);
     if (s != GD_OK) return s;

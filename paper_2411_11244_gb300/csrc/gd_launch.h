@@ -170,6 +170,8 @@ cudaError_t launch_point(PointArgs g, int sms, cudaStream_t stream);
 // co-resident CTAs per SM of the query kernel's single-query or batch launch
 int query_max_blocks_per_sm(int kind, bool batch = false);
 cudaError_t launch_query(int kind, const KArgs& args, int grid, cudaStream_t stream);
+// *best (device): the page of the zeroed buffer that CTA 0's atomics reach soonest
+cudaError_t launch_near_page(unsigned* base, int pages, unsigned words, unsigned* best, int grid, cudaStream_t stream);
 cudaError_t build_query_graph(int kind, const KArgs& args, int grid, cudaGraphExec_t* exec);
 
 }  // namespace gd
