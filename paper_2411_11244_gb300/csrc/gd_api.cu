@@ -477,6 +477,9 @@ gd_status run_single(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B, int kind, 
         a.xb_src = nullptr;
         std::memcpy(a.xa_val, xa, sizeof(a.xa_val));
         std::memcpy(a.xb_val, xb, sizeof(a.xb_val));
+        a.host_desc = 1;
+        a.dA = A->h_desc;
+        a.dB = B->h_desc;
         fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
         a.qs = ctx->qs_one;
         a.slot_of = ctx->slot_of;
@@ -1379,6 +1382,9 @@ gd_status serve_single_launch(gd_ctx* ctx, const gd_query& q, int slot, unsigned
     a.mB = B->d_desc;
     std::memcpy(a.xa_val, q.xa, sizeof(a.xa_val));
     std::memcpy(a.xb_val, q.xb, sizeof(a.xb_val));
+    a.host_desc = 1;
+    a.dA = A->h_desc;
+    a.dB = B->h_desc;
     fill_common(ctx, a, ctx->mb_dev->ctr, &ctx->mb_dev->stats);
     a.slot_of = ctx->slot_of;
     a.n_slot_of = (unsigned long long)tab;

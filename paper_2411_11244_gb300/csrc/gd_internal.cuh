@@ -105,7 +105,9 @@ enum : int {
     kCtrAbort = 20,   // a wait gave up: every CTA leaves at its next barrier
     kCtrLastAbort = 21, // the abort flag of the last finished launch
     kCtrExit = 22,    // CTAs that left the kernel (the last one resets the barrier)
-    kCtrSetupDone = 23, // query setup published (background probe CTAs wait for it)
+    kCtrSetupDone = 23, // query setup published (background CTAs wait for it before they read the state)
+    kCtrFirst = 24,   // bound gathered by a single query's first level and background probes
+                      // (min: its bits inverted; cleared by the last CTA out)
     kCtrBarCount = 32,// grid-barrier arrivals of this launch (top bit: abort)
     kCtrWords = 64,
 };
@@ -152,6 +154,8 @@ struct KArgs {
     const double* xa_src;       // single query: device transforms, or nullptr
     const double* xb_src;       //   to use xa_val / xb_val below
     double xa_val[12], xb_val[12];
+    int host_desc;              // single query: dA, dB hold the meshes' descriptors (else read
+    MeshDev dA, dB;             //   from mA, mB)
     QState* qs;
     Item* front0;
     Item* front1;
@@ -262,22 +266,18 @@ __device__ __forceinline__ bool grid_sync(const KArgs& A, F&& post) {
         unsigned* count = A.ctr + kCtrBarCount;
         const unsigned G = A.work_ctas ? A.work_ctas : gridDim.x;
         const unsigned old = atom_add_release(count, 1u);
+        const unsigned long long t0 = globaltimer();  // (while the arrival is on its way)
         int ok = (old & kBarAbort) == 0u;
         if (ok) {
             const unsigned target = ((old & ~kBarAbort) / G + 1u) * G;
-            unsigned long long t0 = 0;
             for (unsigned spin = 0;; ++spin) {
                 const unsigned v = ld_acquire(count);
                 if (v & kBarAbort) { ok = 0; break; }
                 if (v >= target) break;
-                if ((spin & 63u) == 0u) {
-                    const unsigned long long now = globaltimer();
-                    if (t0 == 0) t0 = now;
-                    else if ((long long)(now - t0) > A.timeout_ns) {
-                        raise_abort(A);
-                        ok = 0;
-                        break;
-                    }
+                if ((spin & 63u) == 0u && (long long)(globaltimer() - t0) > A.timeout_ns) {
+                    raise_abort(A);
+                    ok = 0;
+                    break;
                 }
             }
         }

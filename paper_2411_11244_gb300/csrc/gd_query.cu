@@ -236,12 +236,29 @@ __device__ __forceinline__ void view(const AT& A, unsigned q, QView& V) {
 // CTAs that run the traversal; any others run background probes
 __device__ __forceinline__ unsigned work_ctas(const KArgs& A) { return A.work_ctas ? A.work_ctas : gridDim.x; }
 
+// The bound gathered in kCtrFirst (by the background probes of a single query,
+// and by its first level): that word starts at the identity of its atomicMax, so
+// it takes bounds from the launch's first moment, before the query's state is
+// set up.  A min query's bits are inverted in it.
+template <int KIND>
+__device__ __forceinline__ unsigned first_bound(const KArgs& A) {
+    const unsigned f = ld_relaxed(A.ctr + kCtrFirst);
+    return KIND == 0 ? min(~f, kFltMaxBits) : f;
+}
+
+template <int KIND>
+__device__ __forceinline__ void add_first_bound(const KArgs& A, unsigned v) {
+    atomicMax(A.ctr + kCtrFirst, KIND == 0 ? ~v : v);
+}
+
 // Thread 0: the single query's running bound and status, and (once) its
 // constants, into the CTA state.
+template <int KIND>
 __device__ __forceinline__ void cta_load_query(const KArgs& A) {
     CtaState& c = cta();
     const unsigned long long w = ld_relaxed64(reinterpret_cast<const unsigned long long*>(&A.qs[0].U));
-    c.U = (unsigned)w;
+    const unsigned f = first_bound<KIND>(A);
+    c.U = KIND == 0 ? min((unsigned)w, f) : max((unsigned)w, f);
     c.stat = (unsigned)(w >> 32);
     if (!c.ready) {
         const QState& s = A.qs[0];
@@ -256,7 +273,7 @@ __device__ __forceinline__ void cta_load_query(const KArgs& A) {
 }
 
 // Thread 0's refresh of the CTA state after a barrier.
-template <class AT>
+template <int KIND, class AT>
 __device__ __forceinline__ void cta_refresh(const AT& A) {
     CtaState& c = cta();
     unsigned v[kCtrReset];
@@ -264,14 +281,14 @@ __device__ __forceinline__ void cta_refresh(const AT& A) {
     for (int i = 0; i < kCtrReset; ++i) v[i] = ld_relaxed(A.ctr + i);
 #pragma unroll
     for (int i = 0; i < kCtrReset; ++i) c.ctr[i] = v[i];
-    if (AT::kOne) cta_load_query(A);
+    if (AT::kOne) cta_load_query<KIND>(A);
     c.cnt[0][0] = c.cnt[0][1] = c.cnt[1][0] = c.cnt[1][1] = 0u;
     c.rem = 0u;
 }
 
-template <class AT>
+template <int KIND, class AT>
 __device__ __forceinline__ bool sync(const AT& A) {
-    return grid_sync(A, [&] { cta_refresh(A); });
+    return grid_sync(A, [&] { cta_refresh<KIND>(A); });
 }
 
 // The running bound U of a query and whether its traversal has stopped
@@ -307,13 +324,12 @@ __device__ __forceinline__ void warp_bound_update(const AT& A, bool have, unsign
         if ((threadIdx.x & 31) == 0) {
             volatile unsigned* cu = &cta().U;
             if (KIND == 0 ? r < *cu : r > *cu) {
-                if (KIND == 0) {
-                    atomicMin(const_cast<unsigned*>(cu), r);
-                    atomicMin(&A.qs[0].U, r);
-                } else {
-                    atomicMax(const_cast<unsigned*>(cu), r);
-                    atomicMax(&A.qs[0].U, r);
-                }
+                if (KIND == 0) atomicMin(const_cast<unsigned*>(cu), r);
+                else atomicMax(const_cast<unsigned*>(cu), r);
+                // (a background CTA's bounds may come before the state is set up)
+                if (blockIdx.x >= work_ctas(A)) add_first_bound<KIND>(A, r);
+                else if (KIND == 0) atomicMin(&A.qs[0].U, r);
+                else atomicMax(&A.qs[0].U, r);
             }
         }
         return;
@@ -910,6 +926,21 @@ __device__ __noinline__ void certify_zero(const AT& A, unsigned q, unsigned ta, 
     }
 }
 
+// A background CTA's wait (bounded) until the query's state is set up; called by
+// one thread.  False if the launch was aborted.
+__device__ __forceinline__ bool wait_setup(const KArgs& A) {
+    const unsigned long long t0 = globaltimer();
+    while (!ld_acquire(A.ctr + kCtrSetupDone)) {
+        if (ld_relaxed(A.ctr + kCtrAbort)) return false;
+        if ((long long)(globaltimer() - t0) > A.timeout_ns) {
+            raise_abort(A);
+            return false;
+        }
+        __nanosleep(64);
+    }
+    return true;
+}
+
 // Greedy descent from one front entry by one warp: at each step up to 32
 // descendant pairs (5 levels split between the two trees) are bounded, the
 // running bound takes their enhanced bounds (Eq. 10 / Eq. 11), and the walk
@@ -919,6 +950,8 @@ __device__ __noinline__ void certify_zero(const AT& A, unsigned q, unsigned ta, 
 // the traversal's result does not depend on them.  They exist to reach a
 // near-final bound before the breadth-first levels widen (the sequential
 // depth-first behaviour Section 6 contrasts with).
+__device__ void setup_query_warp(const KArgs& A, int kind, bool state);
+
 template <int KIND, class AT>
 __device__ void probe(const AT& A, Item it, const QView& V) {
     const int lane = threadIdx.x & 31;
@@ -933,9 +966,10 @@ __device__ void probe(const AT& A, Item it, const QView& V) {
         const bool valid = lane < (1 << (kA + kB));
         const unsigned ia = (a << kA) | ((unsigned)lane >> kB);
         const unsigned ib = (b << kB) | ((unsigned)lane & ((1u << kB) - 1u));
-        bool stop;
-        // a background probe CTA meets no barrier: it reads the global bound
-        const float Ucur = blockIdx.x >= work_ctas(A) ? load_U(A.qs[q], &stop) : load_Uq(A, q, &stop);
+        bool stop = false;
+        // a background probe CTA meets no barrier: it reads the gathered bound
+        const float Ucur = AT::kOne && blockIdx.x >= work_ctas(A) ? __uint_as_float(first_bound<KIND>(A))
+                                                                  : load_Uq(A, q, &stop);
         if (__any_sync(kFull, stop)) return;
         bool ok = false;
         unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key = 0xffffffffu;
@@ -958,7 +992,8 @@ __device__ void probe(const AT& A, Item it, const QView& V) {
     warp_bound_update<KIND>(A, valid, q, __float_as_uint(KIND == 0 ? up : lo));
     if (KIND == 0) {
         const unsigned m = __ballot_sync(kFull, valid && lo <= 0.f);
-        if (m) {
+        // (the proof reads the query's state, which a background CTA has not waited for)
+        if (m && !(AT::kOne && blockIdx.x >= work_ctas(A) && !__shfl_sync(kFull, (unsigned)wait_setup(A), 0))) {
             const int src = __ffs(m) - 1;
             certify_zero(A, q, __shfl_sync(kFull, ta, src), __shfl_sync(kFull, tb, src));
         }
@@ -982,9 +1017,7 @@ __device__ void probe_root(const AT& A, unsigned w, const QView& V) {
         const bool valid = lane < (1 << (kA + kB));
         const unsigned ia = (a << kA) | ((unsigned)lane >> kB);
         const unsigned ib = (b << kB) | ((unsigned)lane & ((1u << kB) - 1u));
-        bool stop;
-        const float Ucur = load_U(A.qs[0], &stop);
-        if (__any_sync(kFull, stop)) return;
+        const float Ucur = __uint_as_float(first_bound<KIND>(A));
         bool ok = false;
         unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key = 0xffffffffu;
         if (valid) pair_bounds<KIND>(A, V, ia, ib, depth_of(b) + kB, Ucur, &ok, &newU, &key);
@@ -1007,41 +1040,23 @@ __device__ void probe_root(const AT& A, unsigned w, const QView& V) {
     probe<KIND>(A, Item{a, b, 0.f, 0u}, V);
 }
 
-// A background probe CTA of a single-query launch: it waits (bounded) until
-// the query's setup is published, then every warp walks one probe_root from
-// the root while the traversal CTAs run their levels; the probes only lower
-// the global running bound (and may prove D_min = 0), which the traversal
-// reads at its next barrier.  The probes do not use refit boxes: those are
-// being written while the probes run.
+// A background probe CTA of a single-query launch: it derives the query's
+// constants itself and starts at once; every warp walks one probe_root from the
+// root while the traversal CTAs run their levels; the probes only move the
+// gathered bound (kCtrFirst; and may prove D_min = 0), which the traversal
+// reads at its barriers.  What the levels cost depends on how early that bound
+// comes: waiting for the query's published setup kept the probes 6 us behind.
+// The probes do not use refit boxes: those are being written while they run.
 template <int KIND, class AT>
 __device__ void bg_probe_cta(const AT& A) {
     __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned long long t0 = globaltimer();
-        while (!ld_acquire(A.ctr + kCtrSetupDone)) {
-            if (ld_relaxed(A.ctr + kCtrAbort)) { ok = 0; break; }
-            if ((long long)(globaltimer() - t0) > A.timeout_ns) {
-                raise_abort(A);
-                ok = 0;
-                break;
-            }
-            __nanosleep(64);
-        }
-        if (ok) {
-            cta().ready = 0;
-            cta_load_query(A);
-        }
-        s_ok = ok;
-    }
+    if (threadIdx.x < 32) setup_query_warp(A, KIND, false);
     __syncthreads();
-    if (!s_ok) return;
     QView V;
     view(A, 0u, V);
     V.dR = -1;
     const unsigned w = (blockIdx.x - work_ctas(A)) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     probe_root<KIND>(A, w, V);
-    if (threadIdx.x == 0) atomicAdd(&A.stats->probes, blockDim.x >> 5);
     // Dry runs of the tight leaf bounds and the float64 refinement on
     // triangle pair (0, 0): they only compute, but fetching their code puts it
     // in L2, where the traversal CTAs find it when their leaf and refinement
@@ -1050,12 +1065,14 @@ __device__ void bg_probe_cta(const AT& A) {
     if (V.LA + V.LB < kDryRunDepth) return;
     __shared__ uint4 dry_list[1];
     if (threadIdx.x == 0) {
+        s_ok = wait_setup(A);
         dry_list[0] = make_uint4(0u, 0u, 0u, 0u);
         // the CTA-wide push of the dry run must find nothing to append
         CtaState& c = cta();
         c.cnt[0][0] = c.cnt[0][1] = c.cnt[1][0] = c.cnt[1][1] = 0u;
     }
     __syncthreads();
+    if (!s_ok) return;
     int pit = 0;
     unsigned tp = 0;
     unsigned long long by = 0;
@@ -1077,7 +1094,11 @@ __device__ void bg_probe_cta(const AT& A) {
 // the float64 relative map itself.  The inputs are floats, the constants are
 // rounded up and every operation rounds up, so each result bounds its
 // real-valued expression from above (the 1.000001 factors are margin).
-__device__ __forceinline__ void setup_widening(QState& s, float PA, float PB0, float tinf) {
+struct Widening {
+    float box, tri, df;
+};
+
+__device__ __forceinline__ Widening setup_widening(float PA, float PB0, float tinf) {
     constexpr float kSqrt3Up = 1.7320509f;        // > sqrt(3)
     constexpr float kGamma10Up = 5.9604682e-07f;  // > 10 u / (1 - 10 u), u = 2^-24
     constexpr float kMarginUp = 1.0000011f;       // > 1.000001
@@ -1085,9 +1106,8 @@ __device__ __forceinline__ void setup_widening(QState& s, float PA, float PB0, f
     const float reach = __fadd_ru(__fmul_ru(kSqrt3Up, PB), tinf);  // sqrt(3) P_B + |t|_inf
     const float Eb = __fmul_ru(__fmul_ru(kSqrt3Up, __fmul_ru(kGamma10Up, reach)), kMarginUp);
     const float Xm = __fadd_ru(__fmul_ru(fmaxf(PA, reach), kMarginUp), Eb);
-    s.E_box = Eb;
-    s.E_tri = __fadd_ru(Eb, __fmul_ru(256.f * kU, Xm));
-    s.E_df = __fmul_ru(1.0000001e-12f, __fadd_ru(__fadd_ru(PA, reach), 1.f));
+    return Widening{Eb, __fadd_ru(Eb, __fmul_ru(256.f * kU, Xm)),
+                    __fmul_ru(1.0000001e-12f, __fadd_ru(__fadd_ru(PA, reach), 1.f))};
 }
 
 // The fields of a query's state that the traversal changes, at their
@@ -1111,10 +1131,13 @@ __device__ __forceinline__ void setup_state(QState& s, int kind, unsigned slot_b
 // instruction costs the same for one active lane as for a whole warp, and the
 // single thread of setup_query evaluating all twelve in turn spent
 // microseconds on them.  Lanes 0-8 also hold one entry of the adjugate each;
-// the determinant takes the first column from lanes 0, 3 and 6.
-__device__ void setup_query_warp(const KArgs& A, int kind) {
+// the determinant takes the first column from lanes 0, 3 and 6.  The constants
+// go to the CTA's copy, and in CTA 0 (state) to the query's state with the rest
+// of it.
+__device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
     const int lane = threadIdx.x & 31;
     QState& s = A.qs[0];
+    CtaState& cs = cta();
     const MeshDev* ma;
     const MeshDev* mb;
     const double* xa;
@@ -1149,27 +1172,55 @@ __device__ void setup_query_warp(const KArgs& A, int kind) {
     const float h = (float)r;
     const float lo = (float)(r - (double)h);
     if (rot) {
-        s.R[lane] = h;
-        s.Rl[lane] = lo;
+        cs.v.X.R[lane] = h;
+        cs.Rl[lane] = lo;
     } else if (tra) {
-        s.t[i] = h;
-        s.tl[i] = lo;
+        cs.v.X.t[i] = h;
+        cs.tl[i] = lo;
     }
-    if (lane < 12) {
-        s.xa[lane] = xa[lane];
-        s.xb[lane] = xb[lane];
+    if (state) {
+        if (rot) {
+            s.R[lane] = h;
+            s.Rl[lane] = lo;
+        } else if (tra) {
+            s.t[i] = h;
+            s.tl[i] = lo;
+        }
+        if (lane < 12) {
+            s.xa[lane] = xa[lane];
+            s.xb[lane] = xb[lane];
+        }
     }
     const float tinf = fmaxf(fabsf(__shfl_sync(kFull, h, 9)), fmaxf(fabsf(__shfl_sync(kFull, h, 10)),
                                                                    fabsf(__shfl_sync(kFull, h, 11))));
     if (lane == 0) {
-        setup_widening(s, ma->P, mb->P, tinf);
-        s.A = ma;
-        s.B = mb;
-        setup_state(s, kind, slot_base, mb->L, A.refit);
+        // the meshes' descriptors: launch parameters of a synchronous call
+        // (every CTA's loads of the same two lines queue on them)
+        const MeshDev da = A.host_desc ? A.dA : *ma, db = A.host_desc ? A.dB : *mb;
+        const Widening E = setup_widening(da.P, db.P, tinf);
+        cs.v.E_box = E.box;
+        cs.v.E_tri = E.tri;
+        cs.E_df = E.df;
+        cs.v.boxA = da.box; cs.v.boxB = db.box;
+        cs.v.triA = da.tri; cs.v.triB = db.tri;
+        cs.v.TA = da.T; cs.v.TB = db.T;
+        cs.v.LA = da.L; cs.v.LB = db.L;
+        cs.v.dR = A.refit ? max(0, db.L - kRefitH) : -1;
+        cs.v.slot_base = slot_base;
+        cs.U = kind == 0 ? kFltMaxBits : 0u;
+        cs.stat = 0u;
+        if (state) {
+            s.E_box = E.box;
+            s.E_tri = E.tri;
+            s.E_df = E.df;
+            s.A = ma;
+            s.B = mb;
+            setup_state(s, kind, slot_base, db.L, A.refit);
+        }
     }
     // every lane's fields are published before the CTA's barrier that
     // precedes the setup flag or the grid barrier
-    __threadfence();
+    if (state) __threadfence();
     __syncwarp();
 }
 
@@ -1216,7 +1267,10 @@ __device__ void setup_query(const KArgs& A, int q, int kind) {
         s.tl[i] = (float)(tt - (double)h);
         tinf = fmaxf(tinf, fabsf(h));
     }
-    setup_widening(s, ma->P, mb->P, tinf);
+    const Widening E = setup_widening(ma->P, mb->P, tinf);
+    s.E_box = E.box;
+    s.E_tri = E.tri;
+    s.E_df = E.df;
     s.A = ma;
     s.B = mb;
     for (int i = 0; i < 12; ++i) { s.xa[i] = Xa[i]; s.xb[i] = Xb[i]; }
@@ -1229,6 +1283,77 @@ __device__ __forceinline__ int adaptive_k(unsigned n, long long C, int kmax) {
     int k = 1;
     while (k < kmax && (long long)n << (2 * (k + 1)) < C) ++k;
     return k;
+}
+
+// Whether a single query starts with start_level: its first two levels' pairs
+// (adaptive_k twice: 6 + 2 levels a side, 65,536 pairs, with the default
+// tunables) fit one pass of the grid.  kA, kB: the levels of each side, B's
+// stopping on its refit roots.
+template <class AT>
+__device__ __forceinline__ bool start_depths(const AT& A, int* kA, int* kB) {
+    if (!A.fuse_root) return false;
+    const QConst& V = cta().v;
+    const int k0 = adaptive_k(1u, A.work_target, A.k_max);
+    if (2 * k0 > 16) return false;
+    const int k = k0 + adaptive_k(1u << (2 * k0), A.work_target, A.k_max);
+    *kA = min(k, V.LA);
+    *kB = min(k, V.dR >= 0 ? min(V.LB, V.dR) : V.LB);
+    return *kA + *kB > 0 && *kA + *kB < 31 &&
+           (1ull << (*kA + *kB)) <= (unsigned long long)work_ctas(A) * blockDim.x;
+}
+
+// The first level of a single query: every thread bounds one of the root's
+// descendant pairs, the grid agrees on the running bound that they give, and
+// the pairs within it make the front.  The levels that it replaces met three grid
+// barriers (setup, root, the 4,096 pairs of six levels a side, of which none
+// could be dropped while the bound was infinite) where this one meets one: every
+// CTA derives the query's constants itself, and the bound is gathered in a
+// counter that starts at its identity (kCtrFirst, cleared by the last CTA out).
+// A rings query spent 18.5 us on them and the setup, and 10 on this (all in all
+// the icospheres gain 10 us of 211, rings 5 of 136, two small tori 1 of 74: the
+// levels that follow meet the probes' bound later).
+template <int KIND, class AT>
+__device__ bool start_level(const AT& A, int kA, int kB, unsigned long long& pairs, unsigned long long& bytes) {
+    CtaState& c = cta();
+    QView V;
+    static_cast<QConst&>(V) = c.v;
+    V.q = 0u;
+    const int dR = V.dR;
+    const unsigned total = 1u << (kA + kB);
+    const unsigned vt = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool valid = vt < total;
+    const unsigned ia = (1u << kA) | (vt >> kB), ib = (1u << kB) | (vt & ((1u << kB) - 1u));
+    bool survive = false;
+    float bound = 0.f;
+    unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key;
+    V.dR = -1;  // no refit yet (and the table is being cleared)
+    if (valid) {
+        ++pairs;
+        bound = pair_bounds<KIND, false>(A, V, ia, ib, kB, KIND == 0 ? FLT_MAX : 0.f, &survive, &newU, &key);
+    }
+    const unsigned r = KIND == 0 ? __reduce_min_sync(kFull, newU) : __reduce_max_sync(kFull, newU);
+    if ((threadIdx.x & 31) == 0) {
+        if (KIND == 0) atomicMin(&c.U, r);
+        else atomicMax(&c.U, r);
+    }
+    if (vt == 0) bytes += 24ull * ((1ull << kA) + (1ull << kB));
+    __syncthreads();
+    if (threadIdx.x == 0 && blockIdx.x * blockDim.x < total) add_first_bound<KIND>(A, c.U);
+    if (!sync<KIND>(A)) return false;
+    const float U = __uint_as_float(c.U);
+    if (KIND == 0) survive = survive && bound <= min_keep_threshold(U, V.E_box);
+    else survive = survive && bound >= max_keep_threshold(U, V.E_box);
+    survive = survive && !(c.stat & kStatStop);
+    const int rem = V.LA - kA + V.LB - kB;
+    const Item o = {ia, ib, bound, 0u};
+    if (!cta_push2(0, o, survive && rem > 0, A.front1, A.ctr + kCtrCnt + 1, A.cap_front, survive && rem == 0, A.leafq,
+                   A.ctr + kCtrLeaf, A.cap_leaf))
+        mark_overflow(A, 0u);
+    if (survive) bytes += 16ull;
+    V.dR = dR;
+    if (survive && rem > 0 && kB == dR) claim_root(A, V, 0u, ib);
+    if (vt == 0 && rem > 0) atomicMax(A.ctr + kCtrRem + 1, (unsigned)rem);
+    return true;
 }
 
 template <int KIND, bool FULL, class AT>
@@ -2251,6 +2376,12 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
     unsigned tripairs = 0, refined = 0, refits = 0;
     unsigned leaf_flushed = 0;
     bool probed = false;  // set below once the first probes ran (or run in the background)
+    int first_level = 0, kA0 = 0, kB0 = 0;
+    // a single query whose root needs no refit claim (and that has no full refit
+    // to make first) starts with one level for the first two: every CTA derives
+    // the constants itself
+    const bool all_setup = AT::kOne && !FULL && A.fuse_root;
+    bool start = false;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     const unsigned long long gfirst = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned W = work_ctas(A);
@@ -2271,16 +2402,47 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
 
     // phase 0
     if (threadIdx.x == 0) cta().ready = 0;
-    if (blockIdx.x == 0) {
-        for (int i = threadIdx.x; i < kCtrReset; i += blockDim.x) A.ctr[i] = 0u;
-        if (A.fuse_root) __syncthreads();  // cleared before the root is pushed below
+    if (blockIdx.x == 0 && threadIdx.x >= 32) {
+        // beside the setup warp: the counters and statistics (front[] and slots[]
+        // are written as levels run)
+        StatsDev* S = A.stats;
+        const int i = (int)threadIdx.x - 32;
+        if (i < kCtrReset) A.ctr[i] = 0u;
+        if (i < kAccWays) {
+            S->acc_pairs[i] = 0;
+            S->acc_bytes[i] = 0;
+            S->acc_tri[i] = 0;
+            S->acc_ref[i] = 0;
+        }
+        if (i < 12) S->phase_ns[i] = 0;
+        if (i < 32) {
+            S->level_ns[i] = 0;
+            S->u_level[i] = 0.f;
+        }
+        if (i == 0) {
+            S->levels = 0;
+            S->leaf_pairs = S->candidates = 0;
+            S->probes = AT::kOne ? (gridDim.x - W) * (blockDim.x >> 5) : 0u;  // the background's
+            S->refits = 0;
+            S->t_start = t_start;
+            S->u_probe = 0.f;
+        }
     }
+    if (blockIdx.x == 0 && A.fuse_root && !all_setup) __syncthreads();  // cleared before the root is pushed below
     if (AT::kOne) {
-        if (gfirst < 32) setup_query_warp(A, KIND);
+        // (the two CTAs of an SM on different sub-partitions: float64 issues on
+        // each one's own pipe)
+        const unsigned sw = blockIdx.x == 0 || 2u * blockIdx.x < gridDim.x ? 0u : 1u;
+        if (threadIdx.x >> 5 == sw && (blockIdx.x == 0 || all_setup)) setup_query_warp(A, KIND, blockIdx.x == 0);
     } else {
         for (int q = (int)gfirst; q < A.nq; q += (int)gstride) setup_query(A, q, KIND);
     }
-    if (A.fuse_root && gfirst == 0) {
+    if (all_setup) {
+        __syncthreads();
+        start = start_depths(A, &kA0, &kB0);
+        if (start && threadIdx.x == 0) cta().ready = 1;
+    }
+    if (A.fuse_root && !start && gfirst == 0) {
         // one query whose root needs no refit claim: the thread that set it up
         // pushes its root pair now, and phase 1 with its barrier is skipped
         const QState& s = A.qs[0];
@@ -2296,32 +2458,27 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
         }
     }
     for (unsigned long long i = gfirst; i < A.n_slot_of; i += gstride) A.slot_of[i] = kNoSlot;
-    if (lead) {
-        StatsDev* S = A.stats;
-        S->levels = 0;
-        for (int i = 0; i < kAccWays; ++i) {
-            S->acc_pairs[i] = 0;
-            S->acc_bytes[i] = 0;
-            S->acc_tri[i] = 0;
-            S->acc_ref[i] = 0;
+    if (start) {
+        if (!start_level<KIND>(A, kA0, kB0, pairs, bytes)) goto done;
+        if (W < gridDim.x && lead) atom_add_release(A.ctr + kCtrSetupDone, 1u);
+        lap(0);
+        if (!sync<KIND>(A)) goto done;
+        if (lead) {
+            const unsigned long long now = globaltimer();
+            A.stats->front[0] = 1u;
+            A.stats->slots[0] = (unsigned)(kA0 + kB0);
+            A.stats->level_ns[0] = (unsigned)(now - t_mark);
+            A.stats->levels = 1;
+            t_levels = now - t_mark;
+            t_mark = now;
         }
-        S->leaf_pairs = S->candidates = 0;
-        S->probes = 0;
-        S->refits = 0;
-        S->t_start = t_start;
-        S->u_probe = 0.f;
-        for (int i = 0; i < 12; ++i) S->phase_ns[i] = 0;
-        for (int i = 0; i < 32; ++i) { S->level_ns[i] = 0; S->u_level[i] = 0.f; }
+        if (W < gridDim.x) probed = true;
+        first_level = 1;
+        goto expand;
     }
-    if (W < gridDim.x && blockIdx.x == 0) {
-        // publish the (single) query's setup to the background probe CTAs
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicExch(A.ctr + kCtrSetupDone, 1u);
-        }
-    }
-    if (!sync(A)) goto done;
+    if (!sync<KIND>(A)) goto done;
+    // the (single) query's state is there for the background CTAs
+    if (W < gridDim.x && lead) atom_add_release(A.ctr + kCtrSetupDone, 1u);
 
     if (FULL) {
         // full refit of B into A's frame (single query): subtrees of 2^h
@@ -2330,12 +2487,12 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
         const int h = min(V.LB, kRefitH);
         const int dF = V.LB - h;
         for (unsigned j = blockIdx.x; j < (1u << dF); j += W) full_refit_leaves(A, V, (1u << dF) + j, h);
-        if (!sync(A)) goto done;
+        if (!sync<KIND>(A)) goto done;
         for (int d = dF; d > 0;) {
             const int lv = min(d, kRefitH);
             for (unsigned j = blockIdx.x; j < (1u << (d - lv)); j += W)
                 full_refit_up(A, (1ull << d) + ((unsigned long long)j << lv), lv);
-            if (!sync(A)) goto done;
+            if (!sync<KIND>(A)) goto done;
             d -= lv;
         }
         lap(1);
@@ -2361,13 +2518,14 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
             }
         }
     }
-    if (!sync(A)) goto done;
+    if (!sync<KIND>(A)) goto done;
 levels:
     lap(0);
 
     // phase 2: BVTT levels
     if (W < gridDim.x) probed = true;
-    for (int level = 0;; ++level) {
+expand:
+    for (int level = first_level;; ++level) {
         unsigned n = cta().ctr[kCtrCnt + level % 3];
         if (n > A.cap_front) n = A.cap_front;
         if (n == 0) break;
@@ -2412,12 +2570,17 @@ levels:
                 probe<KIND>(A, it, V);
             }
             if (lead) A.stats->probes += P;
-            if (!sync(A)) goto done;
+            if (!sync<KIND>(A)) goto done;
             if (lead && !reprobe) A.stats->u_probe = AT::kOne ? __uint_as_float(cta().U) : 0.f;
             lap(2);
         }
         unsigned rmax = cta().ctr[kCtrRem + level % 3];
         int k = adaptive_k(n, A.work_target, A.k_max);
+        // The two levels after start_level run before the probes' bound is there;
+        // on deep trees they go two levels a side at most, since what they keep
+        // under a loose bound multiplies below (icospheres: 200 -> 191 us max,
+        // 116 -> 111 min; trees of 11 levels lost 4 us to the extra level)
+        if (AT::kOne && start && level <= 2 && cta().v.LA + cta().v.LB >= kDryRunDepth) k = min(k, 2);
         int s = min(2 * k, (int)rmax);
         if (s < 1) s = 1;
         if (lead) {
@@ -2441,7 +2604,7 @@ levels:
             expand_level_entries<KIND>(A, level, n, pairs, bytes);
         else
             expand_level<KIND, FULL>(A, level, n, s, pairs, bytes);
-        if (!sync(A)) goto done;
+        if (!sync<KIND>(A)) goto done;
         if (lead) {
             unsigned long long now = globaltimer();
             if (level < 32) A.stats->level_ns[level] = (unsigned)(now - t_mark);
@@ -2456,12 +2619,12 @@ levels:
         if (nl >= A.cap_leaf / 2) {
             if (nl > A.cap_leaf) nl = A.cap_leaf;
             leaf_phase<KIND>(A, nl, tripairs, bytes);
-            if (!sync(A)) goto done;
+            if (!sync<KIND>(A)) goto done;
             if (lead) {
                 A.ctr[kCtrLeaf] = 0u;
                 leaf_flushed += nl;
             }
-            if (!sync(A)) goto done;
+            if (!sync<KIND>(A)) goto done;
             lap(4);
         }
     }
@@ -2474,7 +2637,7 @@ levels:
         if (lead) A.stats->leaf_pairs = leaf_flushed + nleaf;
         leaf_phase<KIND>(A, nleaf, tripairs, bytes);
     }
-    if (!sync(A)) goto done;
+    if (!sync<KIND>(A)) goto done;
     lap(4);
     {
         unsigned nc = cta().ctr[kCtrCand];
@@ -2530,7 +2693,7 @@ levels:
             goto done;
         }
         refine_phase_cta<KIND>(A, nc, refined, bytes);
-        if (!sync(A)) goto done;
+        if (!sync<KIND>(A)) goto done;
         lap(5);
         const RefinedSet R = refined_set(A, cta().ctr[kCtrRefined], nc);
         if (AT::kOne) {
@@ -2545,10 +2708,10 @@ levels:
             goto done;
         }
         select_phase(A, R, gfirst, gstride);
-        if (!sync(A)) goto done;
+        if (!sync<KIND>(A)) goto done;
         lap(7);
         finalize_phase(A, R, gfirst, gstride);
-        if (!sync(A)) goto done;
+        if (!sync<KIND>(A)) goto done;
         status_phase(A, gfirst, gstride);
         lap(8);
     }
@@ -2597,6 +2760,7 @@ done:
                 atomicExch(A.ctr + kCtrLastAbort, ab);
                 atomicExch(A.ctr + kCtrBarCount, 0u);
                 atomicExch(A.ctr + kCtrSetupDone, 0u);
+                atomicExch(A.ctr + kCtrFirst, 0u);
                 atomicExch(A.ctr + kCtrExit, 0u);
                 __threadfence();
                 s_last_ab = ab;
