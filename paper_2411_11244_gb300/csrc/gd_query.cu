@@ -492,7 +492,9 @@ __device__ __forceinline__ void claim_root(const KArgs& A, const QView& V, unsig
 // (upper: the best feature pair; lower: the separation of the two triangles
 // along the direction between those closest points, valid for any
 // direction and nearly tight for this one), KIND 1 its max distance.
-template <int KIND>
+// GROUP (min kind): eight neighbouring lanes hold the same pair; lane sub of them
+// takes feature pairs sub, sub + 8, sub + 16, and all get the same bounds.
+template <int KIND, bool GROUP = false>
 __device__ __forceinline__ void tri_bounds_core(const V3<float>* Al, const V3<float>* Bl, float E, float* lo,
                                                 float* up) {
     if (KIND == 0) {
@@ -502,17 +504,33 @@ __device__ __forceinline__ void tri_bounds_core(const V3<float>* Al, const V3<fl
         // instruction from L2
         V3<float> P = Al[0], Q = Bl[0];
         float d2 = INFINITY;
+        int win = 0;
 #pragma unroll 1
-        for (int f = 0; f < 21; ++f) {
+        for (int f = GROUP ? (int)(threadIdx.x & 7u) : 0; f < 21; f += GROUP ? 8 : 1) {
             V3<float> p, q;
             float e2;
             bool h;
             tri_feature(f, Al, Bl, &p, &q, &e2, &h);
             if (h) {
-                P = p; Q = p; d2 = 0.f;
+                P = p; Q = p; d2 = 0.f; win = f;
                 break;
             }
-            if (e2 < d2) { d2 = e2; P = p; Q = q; }
+            if (e2 < d2) { d2 = e2; P = p; Q = q; win = f; }
+        }
+        if (GROUP) {
+            // the least (d2, feature) of the eight: feature f was lane f mod 8's
+            float b2 = d2;
+            int bf = win;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                const float o2 = __shfl_xor_sync(kFull, b2, o);
+                const int of = __shfl_xor_sync(kFull, bf, o);
+                if (o2 < b2 || (o2 == b2 && of < bf)) { b2 = o2; bf = of; }
+            }
+            const int src = (int)(threadIdx.x & 24u) | (bf & 7);
+            d2 = b2;
+            P = mk3(__shfl_sync(kFull, P.x, src), __shfl_sync(kFull, P.y, src), __shfl_sync(kFull, P.z, src));
+            Q = mk3(__shfl_sync(kFull, Q.x, src), __shfl_sync(kFull, Q.y, src), __shfl_sync(kFull, Q.z, src));
         }
         *up = upper_from_sq(d2, E);
         float l = 0.f;
@@ -567,7 +585,7 @@ __device__ __forceinline__ void tri_pair_bounds(const QView& V, unsigned ta, uns
 // leaves more than ~u times the pair's local extent (plus E_df) of error.
 // Used for pairs that pass the float32 test, so that only near-ties reach the
 // float64 refinement; it stays on the float32 pipe (float64 is slow here).
-template <int KIND, class AT>
+template <int KIND, bool GROUP, class AT>
 __device__ __forceinline__ void tri_pair_bounds_tight(const AT& A, unsigned q, const QView& V, const Tri32& TA,
                                                       const Tri32& TB, float* lo, float* up) {
     float Rl[9], tl[3], Edf;
@@ -606,7 +624,7 @@ __device__ __forceinline__ void tri_pair_bounds_tight(const AT& A, unsigned q, c
         Bl[k] = mk3(c[0], c[1], c[2]);
         X = fmaxf(X, fmaxf(max_abs3(Al[k]), max_abs3(Bl[k])));
     }
-    tri_bounds_core<KIND>(Al, Bl, __fadd_ru(Edf, __fmul_ru(256.0f * kU * 1.001f, X)), lo, up);
+    tri_bounds_core<KIND, GROUP>(Al, Bl, __fadd_ru(Edf, __fmul_ru(256.0f * kU * 1.001f, X)), lo, up);
 }
 
 // Whether the plane of triangle P separates it from triangle Q by more than
@@ -899,6 +917,10 @@ template <int KIND, class AT>
 __device__ __noinline__ void leaf_tight(const AT& A, const uint4* list, unsigned n, int& pit, unsigned& tripairs,
                                         unsigned long long& bytes, bool dry);
 
+template <class AT>
+__device__ __noinline__ void leaf_tight_group(const AT& A, const uint4* list, unsigned n, int& pit, unsigned& tripairs,
+                                              unsigned long long& bytes, bool dry);
+
 // Proof of D_min = 0 (min kind), run by a whole warp on one pair (ta, tb) of
 // query q whose float32 lower bound is 0: the float64 distance of the pair,
 // computed exactly as the refinement does.  If it is exactly 0 the query is
@@ -1076,6 +1098,7 @@ __device__ void bg_probe_cta(const AT& A) {
     int pit = 0;
     unsigned tp = 0;
     unsigned long long by = 0;
+    if constexpr (KIND == 0) leaf_tight_group(A, dry_list, 1u, pit, tp, by, true);
     leaf_tight<KIND>(A, dry_list, 1u, pit, tp, by, true);
     V3<double> P, Q;
     int ia, ib;
@@ -1602,6 +1625,35 @@ __device__ __forceinline__ void cta_merge_bound(unsigned long long w) {
     if (st) atomicOr(&c.stat, st);
 }
 
+// What follows the tight bounds of the threads' pairs (every thread calls, for
+// the CTA-wide push): running-bound update, candidates, and the D = 0 check of a
+// pair that may touch.
+template <int KIND, class AT>
+__device__ __forceinline__ void leaf_emit(const AT& A, unsigned q, unsigned ta, unsigned tb, float cb, bool have,
+                                          bool emit, unsigned newU, int& pit, unsigned long long& bytes, bool dry) {
+    if (dry) {
+        // keep the result live so that the bounds are computed, then run the
+        // rest with nothing to publish (no bound, no candidate, no D = 0 check)
+        if (have && cb == 1.2345678e-30f) bytes += 1ull;
+        have = false;
+        emit = false;
+    }
+    warp_bound_update<KIND>(A, have, q, newU);
+    Cand c = {ta, tb, cb, q};
+    if (!cta_push2(pit++, c, emit, A.cand, A.ctr + kCtrCand, A.cap_cand, false, (Cand*)nullptr, (unsigned*)nullptr,
+                   0u))
+        mark_overflow(A, q);
+    if (emit) bytes += 16ull;
+    if (KIND == 0) {
+        // a pair that may touch: try to prove D_min = 0 with it
+        const unsigned m = __ballot_sync(kFull, emit && cb <= 0.f);
+        if (m) {
+            const int src = __ffs(m) - 1;
+            certify_zero(A, __shfl_sync(kFull, q, src), __shfl_sync(kFull, ta, src), __shfl_sync(kFull, tb, src));
+        }
+    }
+}
+
 // Tight bounds of the triangle pairs queued in the CTA's list (thread i takes
 // entry i < n; every thread calls, for the CTA-wide push): running-bound
 // update, candidates, and the D = 0 check of a pair that may touch.  One
@@ -1630,7 +1682,7 @@ __device__ __noinline__ void leaf_tight(const AT& A, const uint4* list, unsigned
             if (dry || tri_pair_may_hold<KIND>(V, TA, TB, Ucur, !AT::kOne)) {
                 ++tripairs;
                 float lo, up;
-                tri_pair_bounds_tight<KIND>(A, q, V, TA, TB, &lo, &up);
+                tri_pair_bounds_tight<KIND, false>(A, q, V, TA, TB, &lo, &up);
                 have = true;
                 if (KIND == 0) {
                     newU = __float_as_uint(up);
@@ -1644,27 +1696,43 @@ __device__ __noinline__ void leaf_tight(const AT& A, const uint4* list, unsigned
             }
         }
     }
-    if (dry) {
-        // keep the result live so that the bounds are computed, then run the
-        // rest with nothing to publish (no bound, no candidate, no D = 0 check)
-        if (have && cb == 1.2345678e-30f) bytes += 1ull;
-        have = false;
-        emit = false;
-    }
-    warp_bound_update<KIND>(A, have, q, newU);
-    Cand c = {ta, tb, cb, q};
-    if (!cta_push2(pit++, c, emit, A.cand, A.ctr + kCtrCand, A.cap_cand, false, (Cand*)nullptr, (unsigned*)nullptr,
-                   0u))
-        mark_overflow(A, q);
-    if (emit) bytes += 16ull;
-    if (KIND == 0) {
-        // a pair that may touch: try to prove D_min = 0 with it
-        const unsigned m = __ballot_sync(kFull, emit && cb <= 0.f);
-        if (m) {
-            const int src = __ffs(m) - 1;
-            certify_zero(A, __shfl_sync(kFull, q, src), __shfl_sync(kFull, ta, src), __shfl_sync(kFull, tb, src));
+    leaf_emit<KIND>(A, q, ta, tb, cb, have, emit, newU, pit, bytes, dry);
+}
+
+// The same for a single min query's list of at most kBlock / 8 pairs, which is
+// what most of its CTAs have: eight lanes take an entry and about three features
+// each, where one thread's 21 features in turn were the longest chain of the
+// leaf phase.
+template <class AT>
+__device__ __noinline__ void leaf_tight_group(const AT& A, const uint4* list, unsigned n, int& pit, unsigned& tripairs,
+                                              unsigned long long& bytes, bool dry) {
+    QView V;
+    view(A, 0u, V);
+    bool have = false, emit = false;
+    float cb = 0.f;
+    unsigned newU = 0xffffffffu;
+    unsigned ta = 0u, tb = 0u;
+    // warp w holds entries 4 w .. 4 w + 3 (every lane of it runs the shuffles;
+    // groups beyond the list bound its last entry once more)
+    if ((threadIdx.x & ~31u) >> 3 < n) {
+        const unsigned at = threadIdx.x >> 3;
+        const uint4 e = list[min(at, n - 1u)];
+        ta = e.x;
+        tb = e.y;
+        bool stop;
+        const float Ucur = load_Uq(A, 0u, &stop);
+        const Tri32 TA = load_tri(V.triA, ta), TB = load_tri(V.triB, tb);
+        float lo, up;
+        tri_pair_bounds_tight<0, true>(A, 0u, V, TA, TB, &lo, &up);
+        if (at < n && (threadIdx.x & 7u) == 0u && (dry || !stop)) {
+            ++tripairs;
+            have = true;
+            newU = __float_as_uint(up);
+            cb = lo;
+            emit = lo <= fminf(Ucur, up);
         }
     }
+    leaf_emit<0>(A, 0u, ta, tb, cb, have, emit, newU, pit, bytes, dry);
 }
 
 // The CTA's list of triangle pairs waiting for their tight bounds (both
@@ -1784,6 +1852,13 @@ __device__ void leaf_phase_slots(const AT& A, unsigned nleaf, unsigned& tripairs
     }
     __syncthreads();
     const unsigned n = list_n;
+    if constexpr (KIND == 0 && AT::kOne) {
+        if (n > 0u && n <= (unsigned)kBlock / 8u) {
+            leaf_tight_group(A, list, n, pit, tripairs, bytes, false);
+            __syncthreads();
+            return;
+        }
+    }
     if (n > 0u) leaf_tight<KIND>(A, list, n, pit, tripairs, bytes, false);
     __syncthreads();
 }
