@@ -81,6 +81,7 @@ struct gd_ctx {
     HostDone* hd = nullptr;      // pinned result records, written by the kernel: [0] for the
                                  // synchronous calls, [1..kPipe] for the server's pipelined launches
     unsigned long long hd_seq = 0;
+    unsigned long long last_sync_seq = 0;  // the last synchronous query whose launch may still be leaving
     QState* qs = nullptr;
     QIn* qin_dev = nullptr;
     QIn* qin_host = nullptr;
@@ -370,6 +371,24 @@ int single_fuse_root(const gd_ctx* c, const gd_mesh* B) {
     return (c->tun.refit_mode != 1 || B->L > kRefitH) ? 1 : 0;
 }
 
+// A synchronous query returns when its record is there; its launch may still be
+// leaving, and resets the counters last.  Work for another stream that uses the
+// context's buffers waits for that (a few microseconds, without a CUDA call: the
+// caller's stream may be under capture).
+gd_status wait_left(gd_ctx* c, cudaStream_t st) {
+    if (st == c->stream || !c->hd || c->last_sync_seq == 0) return GD_OK;
+    const volatile unsigned long long* left = &c->hd->exit_seq;
+    const auto t0 = std::chrono::steady_clock::now();
+    for (unsigned spin = 1; *left != c->last_sync_seq; ++spin) {
+        if ((spin & 1023u) == 0u && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(10)) {
+            GD_CUDA(c, cudaStreamSynchronize(c->stream));
+            break;
+        }
+    }
+    c->last_sync_seq = 0;
+    return GD_OK;
+}
+
 // CTAs of a single-query launch that run the traversal: the others (one per
 // 8 probes, at most 1/8 of the grid) run the greedy probes in the background.
 unsigned single_work_ctas(const gd_ctx* c, int grid) {
@@ -498,6 +517,7 @@ gd_status run_single(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B, int kind, 
         a.host_done = ctx->hd;
         a.seq = seq;
         GD_CUDA(ctx, launch_query(kind, a, grid, ctx->stream));
+        ctx->last_sync_seq = seq;
         const volatile unsigned long long* stamp = &ctx->hd->seq;
         bool got = false;
         for (unsigned spin = 1;; ++spin) {
@@ -1168,6 +1188,8 @@ GD_API gd_status gd_query_device(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B
     s = full_refit_tree(ctx, B, a);
     if (s != GD_OK) return s;
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
+    s = wait_left(ctx, st);
+    if (s != GD_OK) return s;
     int grid = grid_blocks(ctx, (int)kind);
     a.work_ctas = single_work_ctas(ctx, grid);
     a.fuse_root = single_fuse_root(ctx, B);
@@ -1260,7 +1282,10 @@ GD_API gd_status gd_graph_launch(gd_graph* g, void* stream) {
         gd_status s = graph_build(g);
         if (s != GD_OK) return s;
     }
-    GD_CUDA(ctx, cudaGraphLaunch(g->exec, stream ? (cudaStream_t)stream : ctx->stream));
+    cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
+    gd_status s = wait_left(ctx, st);
+    if (s != GD_OK) return s;
+    GD_CUDA(ctx, cudaGraphLaunch(g->exec, st));
     ctx->stats_pending = true;
     return GD_OK;
 }

@@ -108,6 +108,7 @@ enum : int {
     kCtrSetupDone = 23, // query setup published (background CTAs wait for it before they read the state)
     kCtrFirst = 24,   // bound gathered by a single query's first level and background probes
                       // (min: its bits inverted; cleared by the last CTA out)
+    kCtrSent = 25,    // CTA 0 has sent a single query's record to the host
     kCtrBarCount = 32,// grid-barrier arrivals of this launch (top bit: abort)
     kCtrWords = 64,
 };
@@ -137,13 +138,16 @@ struct StatsDev {
     unsigned long long t_start;  // globaltimer at the launch's start (CTA 0)
 };
 
-// Result record of a single query in pinned host memory, written by the
-// launch's last CTA (the host polls seq instead of copying and synchronising)
+// Result record of a single query in pinned host memory, written by CTA 0 (by
+// the launch's last CTA for a batch, and for a launch that gave up; the host
+// polls seq instead of copying and synchronising)
 struct HostDone {
     gd_result out;
     unsigned last_abort;          // the launch's abort flag
     unsigned bad_index;           // sites of failed index checks
     unsigned long long seq;       // written last: the launch's sequence number
+    unsigned long long exit_seq;  // ... once the launch has reset its counters (a single query's
+                                  // record comes before that)
 };
 
 struct KArgs {

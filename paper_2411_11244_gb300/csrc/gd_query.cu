@@ -2403,6 +2403,29 @@ __device__ void status_phase(const KArgs& A, unsigned long long first, unsigned 
     }
 }
 
+// A single query's record to the host, by CTA 0 as soon as it is final (every
+// thread calls; the record was written by this CTA before a __syncthreads): the
+// other CTAs' way out and the last one's bookkeeping, about 3 us, are not
+// waited for.  The last CTA out then only stamps HostDone::exit_seq.
+__device__ __forceinline__ void publish_record(const KArgs& A) {
+    if (!A.host_done || A.host_out) return;
+    HostDone* h = A.host_done;
+    static_assert(sizeof(gd_result) % 8 == 0, "result record copied in 8-byte words");
+    constexpr int kW = (int)(sizeof(gd_result) / 8);
+    if (threadIdx.x < kW)
+        reinterpret_cast<unsigned long long*>(&h->out)[threadIdx.x] =
+            __ldcg(reinterpret_cast<const unsigned long long*>(A.out) + threadIdx.x);
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        h->last_abort = 0u;
+        h->bad_index = ld_relaxed(A.ctr + kCtrBadIndex);
+        __threadfence_system();
+        *reinterpret_cast<volatile unsigned long long*>(&h->seq) = A.seq;
+        A.ctr[kCtrSent] = 1u;  // (this thread's exit count releases it to the last CTA)
+    }
+}
+
 // Run the refit jobs appended since the last call (one job per CTA at a time);
 // returns false if the grid barrier after them failed; *ran tells whether
 // there were any.
@@ -2762,6 +2785,7 @@ expand:
                     }
                     status_phase(A, threadIdx.x, blockDim.x);
                     __syncthreads();
+                    if (AT::kOne) publish_record(A);
                     lap(8);
                 }
             }
@@ -2778,6 +2802,8 @@ expand:
                 select_finalize_single(A, R);
                 lap(7);
                 status_phase(A, threadIdx.x, blockDim.x);
+                __syncthreads();
+                publish_record(A);
                 lap(8);
             }
             goto done;
@@ -2816,7 +2842,7 @@ done:
             atomicAdd(&s_tri, tripairs);
             atomicAdd(&s_ref, refined);
         }
-        __shared__ unsigned s_last_ab;
+        __shared__ unsigned s_last_ab, s_sent;
         __shared__ int s_last;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -2836,6 +2862,7 @@ done:
                 atomicExch(A.ctr + kCtrBarCount, 0u);
                 atomicExch(A.ctr + kCtrSetupDone, 0u);
                 atomicExch(A.ctr + kCtrFirst, 0u);
+                s_sent = atomicExch(A.ctr + kCtrSent, 0u);
                 atomicExch(A.ctr + kCtrExit, 0u);
                 __threadfence();
                 s_last_ab = ab;
@@ -2847,10 +2874,11 @@ done:
             // them, were fenced before their exit count): the records go to
             // the host's pinned memory, then the stamp
             HostDone* h = A.host_done;
-            static_assert(sizeof(gd_result) % 8 == 0, "result record copied in 8-byte words");
             constexpr int kW = (int)(sizeof(gd_result) / 8);
             const unsigned long long* src = reinterpret_cast<const unsigned long long*>(A.out);
-            if (A.host_out) {
+            if (s_sent) {
+                // CTA 0 has sent the record
+            } else if (A.host_out) {
                 unsigned long long* dst = reinterpret_cast<unsigned long long*>(A.host_out);
                 for (long long k = threadIdx.x; k < (long long)A.nq * kW; k += blockDim.x) dst[k] = __ldcg(src + k);
             } else if (threadIdx.x < kW) {
@@ -2859,10 +2887,13 @@ done:
             __threadfence_system();
             __syncthreads();
             if (threadIdx.x == 0) {
-                h->last_abort = s_last_ab;
-                h->bad_index = ld_relaxed(A.ctr + kCtrBadIndex);
-                __threadfence_system();
-                *reinterpret_cast<volatile unsigned long long*>(&h->seq) = A.seq;
+                *reinterpret_cast<volatile unsigned long long*>(&h->exit_seq) = A.seq;
+                if (!s_sent) {
+                    h->last_abort = s_last_ab;
+                    h->bad_index = ld_relaxed(A.ctr + kCtrBadIndex);
+                    __threadfence_system();
+                    *reinterpret_cast<volatile unsigned long long*>(&h->seq) = A.seq;
+                }
             }
         }
     }
