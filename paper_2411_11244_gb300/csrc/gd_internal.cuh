@@ -56,6 +56,22 @@ struct QIn {
     unsigned pad;
 };
 
+// The constants of a query of a batch that its levels and leaf phase read for
+// every entry, in the order in which they load them (16 bytes at a time).
+struct __align__(16) QPack {
+    float E_box;
+    int LA, LB;
+    int dR;
+    const float* boxA;
+    const float* boxB;
+    unsigned slot_base;
+    unsigned TA, TB;              // triangles
+    unsigned pad;
+    const float4* triA;
+    const float4* triB;
+    float R[9], t[3];             // B-local -> A-local, float32
+};
+
 // per-query running state and derived constants
 struct __align__(16) QState {
     unsigned U;                   // running bound, float bits (min: upper of
@@ -74,6 +90,7 @@ struct __align__(16) QState {
     int dR;                       // depth of B's refit roots (L_B - min(L_B, kRefitH)), -1: no refit
     unsigned cert;                // float64 intersection checks started (min kind)
     unsigned pushed[2];           // batch: entries pushed at the current level (by parity)
+    QPack pk;                     // batch: what every entry reads
 };
 
 // kStatZero: a pair at float64 distance exactly 0 is a candidate, so D_min = 0

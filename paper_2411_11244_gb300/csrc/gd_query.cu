@@ -24,6 +24,7 @@
 //   6  witness points and result records.
 #include <cfloat>
 #include <cstdio>
+#include <type_traits>
 
 #include "gd_geom.cuh"
 #include "gd_internal.cuh"
@@ -181,6 +182,37 @@ struct QView : QConst {
     unsigned q = 0xffffffffu;
 };
 
+// What a level of a batch reads of an entry's query: loaded for every entry (L1
+// hits) and not kept, since neighbouring entries belong to different queries
+// and a whole QView, refilled at every change, lived in local memory under the
+// batch's 64 registers.  The map itself is loaded only for pairs without a refit box.
+struct BView {
+    const QPack* k;
+    const float* boxA;
+    const float* boxB;
+    float E_box;
+    int LA, LB, dR;
+    unsigned slot_base;
+};
+
+// ... and what its leaf phase reads
+struct LeafView {
+    Rigid32 X;
+    float E_box;
+    int LA, LB;
+    const float4* triA;
+    const float4* triB;
+    long long TA, TB;
+};
+
+__device__ __forceinline__ const Rigid32& map_of(const QView& V) { return V.X; }
+__device__ __forceinline__ Rigid32 map_of(const QPack* k) {
+    const float4* m = reinterpret_cast<const float4*>(k->R);
+    const float4 a = m[0], b = m[1], c = m[2];
+    return Rigid32{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x}, {c.y, c.z, c.w}};
+}
+__device__ __forceinline__ Rigid32 map_of(const BView& V) { return map_of(V.k); }
+
 // Per-CTA shared copies of global state, refreshed by thread 0 right after
 // every grid barrier (the barrier's closing __syncthreads publishes them):
 // the counters, and in a single-query launch the query's constants and its
@@ -231,6 +263,37 @@ __device__ __forceinline__ void view(const AT& A, unsigned q, QView& V) {
     if (AT::kOne) static_cast<QConst&>(V) = cta().v;
     else load_qconst(A.qs[q], V);
     V.q = q;
+}
+
+template <class AT>
+__device__ __forceinline__ void view(const AT& A, unsigned q, BView& V) {
+    const QPack* k = &A.qs[q].pk;
+    const float4 a = *reinterpret_cast<const float4*>(&k->E_box);
+    const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&k->boxA);
+    V.k = k;
+    V.E_box = a.x;
+    V.LA = __float_as_int(a.y);
+    V.LB = __float_as_int(a.z);
+    V.dR = __float_as_int(a.w);
+    V.boxA = reinterpret_cast<const float*>(b.x);
+    V.boxB = reinterpret_cast<const float*>(b.y);
+    V.slot_base = k->slot_base;
+}
+
+template <class AT>
+__device__ __forceinline__ void view(const AT& A, unsigned q, LeafView& V) {
+    const QPack* k = &A.qs[q].pk;
+    const float4 a = *reinterpret_cast<const float4*>(&k->E_box);
+    const uint4 c = *reinterpret_cast<const uint4*>(&k->slot_base);
+    const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(&k->triA);
+    V.E_box = a.x;
+    V.LA = __float_as_int(a.y);
+    V.LB = __float_as_int(a.z);
+    V.TA = c.y;
+    V.TB = c.z;
+    V.triA = reinterpret_cast<const float4*>(d.x);
+    V.triB = reinterpret_cast<const float4*>(d.y);
+    V.X = map_of(k);
 }
 
 // CTAs that run the traversal; any others run background probes
@@ -456,21 +519,24 @@ __device__ __forceinline__ bool cta_push4(int it, const E* v, unsigned m, bool t
 // written, and the refit jobs run beside the next level's expansion (no grid
 // barrier between them): the acquire load makes the boxes visible with the
 // index; a root still being refit reads as kNoSlot (mapped local boxes).
-__device__ __forceinline__ unsigned refit_slot(const KArgs& A, const QView& V, unsigned b, int db) {
+template <class VT>
+__device__ __forceinline__ unsigned refit_slot(const KArgs& A, const VT& V, unsigned b, int db) {
     if (V.dR < 0 || db < V.dR) return kNoSlot;
     unsigned root = b >> (db - V.dR);
     unsigned s = ld_acquire(A.slot_of + V.slot_base + (root - (1u << V.dR)));
     return s < A.cap_slots ? s : kNoSlot;
 }
 
-__device__ __forceinline__ unsigned long long refit_index(const QView& V, unsigned slot, unsigned b, int db) {
+template <class VT>
+__device__ __forceinline__ unsigned long long refit_index(const VT& V, unsigned slot, unsigned b, int db) {
     int rel = db - V.dR;
     unsigned local = (1u << rel) | (b & ((1u << rel) - 1u));
     return (unsigned long long)slot * kRefitBoxes + local;
 }
 
 // Claim the refit of root b for query q (first claimer appends the job).
-__device__ __forceinline__ void claim_root(const KArgs& A, const QView& V, unsigned q, unsigned b) {
+template <class VT>
+__device__ __forceinline__ void claim_root(const KArgs& A, const VT& V, unsigned q, unsigned b) {
     unsigned* e = A.slot_of + V.slot_base + (b - (1u << V.dR));
     if (ld_relaxed(e) != kNoSlot) return;
     if (atomicCAS(e, kNoSlot, kClaimed) != kNoSlot) return;
@@ -714,22 +780,23 @@ __device__ __forceinline__ bool tri_pair_may_hold(const QConst& V, const Tri32& 
 // bound of the max) and whether the pair survives against Ucur; for a
 // survivor, *newU is its enhanced bound (Eq. 10 / Eq. 11) for the running
 // bound and *key orders survivors by it.
-template <int KIND, bool FULL = false>
-__device__ __forceinline__ float pair_bounds(const KArgs& A, const QView& V, unsigned ia, unsigned ib, int db,
-                                             float Ucur, bool* survive, unsigned* newU, unsigned* key) {
+// slot: B's refit slot (refit_slot), looked up by the caller.
+template <int KIND, bool FULL, class VT>
+__device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
+                                                unsigned slot, float Ucur, bool* survive, unsigned* newU,
+                                                unsigned* key) {
     Box ba = load_box(V.boxA, ia);
-    // FULL: B's whole tree was refit into A's frame at the start of the launch
-    const unsigned slot = FULL ? 0u : refit_slot(A, V, ib, db);
     float bound;
     *key = 0xffffffffu;
     if (slot != kNoSlot) {
-        // B's box already in A's frame (refit): plain AABB-AABB bounds
+        // B's box already in A's frame (refit): plain AABB-AABB bounds (no map)
+        const Rigid32 none{};
         Box bb = FULL ? load_box_cg(A.ftree, ib) : load_box_cg(A.rbox, refit_index(V, slot, ib, db));
         if (KIND == 0) {
             bound = lower_min_sq(ba, bb.lo, bb.hi);
             *survive = bound <= min_keep_threshold(Ucur, V.E_box);
             if (*survive) {
-                float u2 = A.conventional ? upper_max_sq(ba, bb.lo, bb.hi) : upper_min_sq_enhanced<true>(V.X, ba, bb);
+                float u2 = A.conventional ? upper_max_sq(ba, bb.lo, bb.hi) : upper_min_sq_enhanced<true>(none, ba, bb);
                 *newU = __float_as_uint(upper_from_sq(u2, V.E_box));
                 *key = __float_as_uint(u2);
             }
@@ -737,20 +804,21 @@ __device__ __forceinline__ float pair_bounds(const KArgs& A, const QView& V, uns
             bound = upper_max_sq(ba, bb.lo, bb.hi);
             *survive = bound >= max_keep_threshold(Ucur, V.E_box);
             if (*survive) {
-                float l2 = A.conventional ? lower_min_sq(ba, bb.lo, bb.hi) : lower_max_sq_enhanced<true>(V.X, ba, bb);
+                float l2 = A.conventional ? lower_min_sq(ba, bb.lo, bb.hi) : lower_max_sq_enhanced<true>(none, ba, bb);
                 *newU = __float_as_uint(lower_from_sq(l2, V.E_box));
                 *key = ~__float_as_uint(l2);
             }
         }
     } else {
         Box bb = load_box(V.boxB, ib);
+        const Rigid32& X = map_of(V);
         float elo[3], ehi[3];
-        enclose(V.X, bb, elo, ehi);
+        enclose(X, bb, elo, ehi);
         if (KIND == 0) {
             bound = lower_min_sq(ba, elo, ehi);
             *survive = bound <= min_keep_threshold(Ucur, V.E_box);
             if (*survive) {
-                float u2 = A.conventional ? upper_max_sq(ba, elo, ehi) : upper_min_sq_enhanced<false>(V.X, ba, bb);
+                float u2 = A.conventional ? upper_max_sq(ba, elo, ehi) : upper_min_sq_enhanced<false>(X, ba, bb);
                 *newU = __float_as_uint(upper_from_sq(u2, V.E_box));
                 *key = __float_as_uint(u2);
             }
@@ -758,13 +826,20 @@ __device__ __forceinline__ float pair_bounds(const KArgs& A, const QView& V, uns
             bound = upper_max_sq(ba, elo, ehi);
             *survive = bound >= max_keep_threshold(Ucur, V.E_box);
             if (*survive) {
-                float l2 = A.conventional ? lower_min_sq(ba, elo, ehi) : lower_max_sq_enhanced<false>(V.X, ba, bb);
+                float l2 = A.conventional ? lower_min_sq(ba, elo, ehi) : lower_max_sq_enhanced<false>(X, ba, bb);
                 *newU = __float_as_uint(lower_from_sq(l2, V.E_box));
                 *key = ~__float_as_uint(l2);
             }
         }
     }
     return bound;
+}
+
+template <int KIND, bool FULL = false, class VT>
+__device__ __forceinline__ float pair_bounds(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
+                                             float Ucur, bool* survive, unsigned* newU, unsigned* key) {
+    // FULL: B's whole tree was refit into A's frame at the start of the launch
+    return pair_bounds_at<KIND, FULL>(A, V, ia, ib, db, FULL ? 0u : refit_slot(A, V, ib, db), Ucur, survive, newU, key);
 }
 
 // ------------------------------------------------------------- refit
@@ -1298,6 +1373,20 @@ __device__ void setup_query(const KArgs& A, int q, int kind) {
     s.B = mb;
     for (int i = 0; i < 12; ++i) { s.xa[i] = Xa[i]; s.xb[i] = Xb[i]; }
     setup_state(s, kind, slot_base, mb->L, A.refit);
+    QPack& k = s.pk;
+    k.E_box = E.box;
+    k.LA = ma->L;
+    k.LB = mb->L;
+    k.dR = s.dR;
+    k.boxA = ma->box;
+    k.boxB = mb->box;
+    k.slot_base = slot_base;
+    k.TA = (unsigned)ma->T;
+    k.TB = (unsigned)mb->T;
+    k.triA = ma->tri;
+    k.triB = mb->tri;
+    for (int i = 0; i < 9; ++i) k.R[i] = s.R[i];
+    for (int i = 0; i < 3; ++i) k.t[i] = s.t[i];
 }
 
 // ------------------------------------------------------------- phase 2
@@ -1391,7 +1480,7 @@ __device__ void expand_level(const AT& A, int level, unsigned n, int s, unsigned
     const unsigned long long gstride = (unsigned long long)work_ctas(A) * blockDim.x;
     const unsigned long long mask = (1ull << s) - 1;
     const int lane = threadIdx.x & 31;
-    QView V;
+    std::conditional_t<AT::kOne, QView, BView> V;
     // CTA-uniform loop: every thread of a CTA runs the same iterations, so
     // that the appends can be counted per CTA (cta_push2)
     int iter = 0;
@@ -1500,7 +1589,7 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
     unsigned* leaf_cnt = A.ctr + kCtrLeaf;
     const unsigned long long gstride = (unsigned long long)work_ctas(A) * blockDim.x;
     const int lane = threadIdx.x & 31;
-    QView V;
+    std::conditional_t<AT::kOne, QView, BView> V;
     int iter = 0;
     for (unsigned long long cbase = (unsigned long long)blockIdx.x * blockDim.x; cbase < n;
          cbase += gstride, ++iter) {
@@ -1544,6 +1633,12 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
         Item o[4];
         unsigned sm = 0u;
         unsigned best = KIND == 0 ? 0xffffffffu : 0u;
+        // B's children lie below one refit root on all levels but the root's own
+        // (kB levels): one look-up, whose acquire the children's loads then wait
+        // for once and not each
+        const bool one_root = V.dR < 0 || dBc < V.dR || dBc - V.dR >= kB;
+        unsigned slot = kNoSlot;
+        if (valid && one_root) slot = refit_slot(A, V, it.b << kB, dBc);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const unsigned ia = (it.a << kA) | ((unsigned)c >> kB);
@@ -1553,7 +1648,8 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
                 ++pairs;
                 bool survive = false;
                 unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key;
-                o[c].bound = pair_bounds<KIND, false>(A, V, ia, ib, dBc, Ucur, &survive, &newU, &key);
+                if (!one_root) slot = refit_slot(A, V, ib, dBc);
+                o[c].bound = pair_bounds_at<KIND, false>(A, V, ia, ib, dBc, slot, Ucur, &survive, &newU, &key);
                 if (survive) {
                     sm |= 1u << c;
                     best = KIND == 0 ? min(best, newU) : max(best, newU);
@@ -1746,10 +1842,12 @@ __device__ __noinline__ void leaf_tight_group(const AT& A, const uint4* list, un
     leaf_emit<0>(A, 0u, ta, tb, cb, have, emit, newU, pit, bytes, dry);
 }
 
-// The CTA's list of triangle pairs waiting for their tight bounds (both
-// forms of the leaf phase use it; it holds 3 kBlock entries).
+// The CTA's list of triangle pairs waiting for their tight bounds: fewer than
+// kBlock between iterations, and one iteration's pairs (one a thread; in a batch
+// up to four).
+template <bool ONE>
 __device__ __forceinline__ uint4* leaf_list() {
-    __shared__ uint4 l[3 * kBlock];
+    __shared__ uint4 l[(ONE ? 2 : 5) * kBlock];
     return l;
 }
 
@@ -1770,7 +1868,7 @@ __device__ void leaf_phase_slots(const AT& A, unsigned nleaf, unsigned& tripairs
     // slots per thread and iteration (two, measured for single queries: the
     // leaf phase took 17.2 -> 18.3 us on the rings; one kept)
     constexpr int U = 1;
-    uint4* list = leaf_list();
+    uint4* list = leaf_list<AT::kOne>();
     unsigned& list_n = leaf_list_n();
     const unsigned long long total = (unsigned long long)nleaf * 4ull;
     const unsigned long long gstride = (unsigned long long)work_ctas(A) * blockDim.x;
@@ -1874,25 +1972,24 @@ __device__ void leaf_phase_slots(const AT& A, unsigned nleaf, unsigned& tripairs
     __syncthreads();
 }
 
-// The same two stages with one thread per leaf pair: it loads the pair's
+// The same two stages with one thread per leaf pair (batches): it loads the pair's
 // (up to) 2 + 2 triangles, maps each of B's into A's frame once, and runs the
-// cheap test on its (up to) four triangle pairs.  The passing pairs reach the
-// list in two pushes of two between CTA barriers, so that it holds fewer
-// than kBlock + 2 kBlock entries before a drain.
+// cheap test on its (up to) four triangle pairs.  A warp reserves the list places
+// of all its passing pairs at once, and the CTA meets one barrier an iteration:
+// each warp knows the list's length after its own push, so the barrier's OR says
+// whether it holds a CTA's worth (with the pairs pushed two a thread between
+// barriers, five an iteration, a gear batch's leaf phases took 6.7 ms for 177 M
+// pairs; this form 6.3).
 template <int KIND, class AT>
 __device__ void leaf_phase_pairs(const AT& A, unsigned nleaf, unsigned& tripairs, unsigned long long& bytes) {
-    uint4* list = leaf_list();
+    uint4* list = leaf_list<AT::kOne>();
     unsigned& list_n = leaf_list_n();
     const unsigned long long gstride = (unsigned long long)work_ctas(A) * blockDim.x;
-    const bool pull = AT::kOne && threadIdx.x == 0;
     const int lane = threadIdx.x & 31;
-    QView Vb;
     int pit = 0;
     if (threadIdx.x == 0) list_n = 0u;
+    __syncthreads();
     for (unsigned long long cbase = (unsigned long long)blockIdx.x * blockDim.x; cbase < nleaf; cbase += gstride) {
-        if (__syncthreads_or(AT::kOne && (((volatile CtaState&)cta()).stat & kStatStop) != 0u)) break;
-        unsigned long long gw = 0;
-        if (pull) gw = ld_relaxed64(reinterpret_cast<const unsigned long long*>(&A.qs[0].U));
         const unsigned long long vt = cbase + threadIdx.x;
         bool valid = vt < nleaf;
         Item it = Item{1u, 1u, 0.f, 0u};
@@ -1906,8 +2003,8 @@ __device__ void leaf_phase_pairs(const AT& A, unsigned nleaf, unsigned& tripairs
             }
         }
         const unsigned q = it.q;
-        if (!AT::kOne) view(A, q, Vb);
-        const QConst& V = AT::kOne ? static_cast<const QConst&>(cta().v) : static_cast<const QConst&>(Vb);
+        LeafView V;
+        view(A, q, V);
         if (valid && (depth_of(it.a) != V.LA || depth_of(it.b) != V.LB)) {
             flag_bad(A, kBadLeaf);
             valid = false;
@@ -1941,31 +2038,32 @@ __device__ void leaf_phase_pairs(const AT& A, unsigned nleaf, unsigned& tripairs
                 if (a2 && tri_pair_may_hold_mapped<KIND>(V.E_box, TA1, Bw, Ucur, true)) m |= 8u;
             }
         }
+        // the warp's places, in the order of the lanes (counts of 0 to 4: three ballots)
+        const unsigned cnt = (unsigned)__popc(m);
+        unsigned pre = 0u, tot = 0u;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int b = 0; b < 3; ++b) {
+            const unsigned w = __ballot_sync(kFull, (cnt >> b) & 1u);
+            pre += (unsigned)__popc(w & lanemask_lt()) << b;
+            tot += (unsigned)__popc(w) << b;
+        }
+        unsigned base = 0u;
+        if (lane == 0) base = atomicAdd(&list_n, tot);
+        const bool full = lane == 0 && base + tot >= (unsigned)kBlock;
+        unsigned to = __shfl_sync(kFull, base, 0) + pre;
 #pragma unroll
-            for (int r = 2 * h; r < 2 * h + 2; ++r) {
-                const bool p = (m >> r) & 1u;
-                const unsigned mb = __ballot_sync(kFull, p);
-                unsigned base = 0u;
-                if (lane == 0 && mb) base = atomicAdd(&list_n, (unsigned)__popc(mb));
-                base = __shfl_sync(kFull, base, 0);
-                if (p) list[base + __popc(mb & lanemask_lt())] = make_uint4(a0 + (r >> 1), b0 + (r & 1), q, 0u);
+        for (int r = 0; r < 4; ++r)
+            if ((m >> r) & 1u) list[to++] = make_uint4(a0 + (r >> 1), b0 + (r & 1), q, 0u);
+        if (__syncthreads_or(full)) {
+            unsigned n = list_n;  // (no push before the barrier at the end)
+            while (n >= (unsigned)kBlock) {
+                leaf_tight<KIND>(A, list + (n - kBlock), kBlock, pit, tripairs, bytes, false);
+                __syncthreads();
+                n -= kBlock;
             }
-            __syncthreads();
-            unsigned n = list_n;
-            if (n >= (unsigned)kBlock) {
-                while (n >= (unsigned)kBlock) {
-                    leaf_tight<KIND>(A, list + (n - kBlock), kBlock, pit, tripairs, bytes, false);
-                    __syncthreads();
-                    n -= kBlock;
-                }
-                if (threadIdx.x == 0) list_n = n;
-            }
-            // every thread has read list_n before the next push changes it
+            if (threadIdx.x == 0) list_n = n;
             __syncthreads();
         }
-        if (pull) cta_merge_bound<KIND>(gw);
     }
     __syncthreads();
     const unsigned n = list_n;
@@ -2474,8 +2572,11 @@ __device__ bool refit_jobs(const AT& A, bool lead, unsigned& refits, bool* ran) 
 // query (nq == 1) or a batch; with the query count known at compile time
 // every single-query / batch branch of the inlined phases folds, so each
 // instantiation carries only its own code and register pressure.
+// CTAs per SM of a batch: 3 (80 registers) once its levels and leaf phase load a
+// query's constants per entry (256 gear queries: 17.5 ms; 4 CTAs 18.1, and
+// 20.7 with the constants kept in registers, which then lived in local memory).
 #ifndef GD_BATCH_CTAS
-#define GD_BATCH_CTAS 4
+#define GD_BATCH_CTAS 3
 #endif
 template <int KIND, bool FULL, bool ONE>
 __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs Aparam) {
