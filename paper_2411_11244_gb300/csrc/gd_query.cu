@@ -1193,7 +1193,7 @@ __device__ void bg_probe_cta(const AT& A) {
 // rounded up and every operation rounds up, so each result bounds its
 // real-valued expression from above (the 1.000001 factors are margin).
 struct Widening {
-    float box, tri, df;
+    float E_box, E_tri, E_df;
 };
 
 __device__ __forceinline__ Widening setup_widening(float PA, float PB0, float tinf) {
@@ -1204,8 +1204,11 @@ __device__ __forceinline__ Widening setup_widening(float PA, float PB0, float ti
     const float reach = __fadd_ru(__fmul_ru(kSqrt3Up, PB), tinf);  // sqrt(3) P_B + |t|_inf
     const float Eb = __fmul_ru(__fmul_ru(kSqrt3Up, __fmul_ru(kGamma10Up, reach)), kMarginUp);
     const float Xm = __fadd_ru(__fmul_ru(fmaxf(PA, reach), kMarginUp), Eb);
-    return Widening{Eb, __fadd_ru(Eb, __fmul_ru(256.f * kU, Xm)),
-                    __fmul_ru(1.0000001e-12f, __fadd_ru(__fadd_ru(PA, reach), 1.f))};
+    Widening s;
+    s.E_box = Eb;
+    s.E_tri = __fadd_ru(Eb, __fmul_ru(256.f * kU, Xm));
+    s.E_df = __fmul_ru(1.0000001e-12f, __fadd_ru(__fadd_ru(PA, reach), 1.f));
+    return s;
 }
 
 // The fields of a query's state that the traversal changes, at their
@@ -1296,9 +1299,9 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
         // (every CTA's loads of the same two lines queue on them)
         const MeshDev da = A.host_desc ? A.dA : *ma, db = A.host_desc ? A.dB : *mb;
         const Widening E = setup_widening(da.P, db.P, tinf);
-        cs.v.E_box = E.box;
-        cs.v.E_tri = E.tri;
-        cs.E_df = E.df;
+        cs.v.E_box = E.E_box;
+        cs.v.E_tri = E.E_tri;
+        cs.E_df = E.E_df;
         cs.v.boxA = da.box; cs.v.boxB = db.box;
         cs.v.triA = da.tri; cs.v.triB = db.tri;
         cs.v.TA = da.T; cs.v.TB = db.T;
@@ -1308,9 +1311,9 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
         cs.U = kind == 0 ? kFltMaxBits : 0u;
         cs.stat = 0u;
         if (state) {
-            s.E_box = E.box;
-            s.E_tri = E.tri;
-            s.E_df = E.df;
+            s.E_box = E.E_box;
+            s.E_tri = E.E_tri;
+            s.E_df = E.E_df;
             s.A = ma;
             s.B = mb;
             setup_state(s, kind, slot_base, db.L, A.refit);
@@ -1366,15 +1369,15 @@ __device__ void setup_query(const KArgs& A, int q, int kind) {
         tinf = fmaxf(tinf, fabsf(h));
     }
     const Widening E = setup_widening(ma->P, mb->P, tinf);
-    s.E_box = E.box;
-    s.E_tri = E.tri;
-    s.E_df = E.df;
+    s.E_box = E.E_box;
+    s.E_tri = E.E_tri;
+    s.E_df = E.E_df;
     s.A = ma;
     s.B = mb;
     for (int i = 0; i < 12; ++i) { s.xa[i] = Xa[i]; s.xb[i] = Xb[i]; }
     setup_state(s, kind, slot_base, mb->L, A.refit);
     QPack& k = s.pk;
-    k.E_box = E.box;
+    k.E_box = E.E_box;
     k.LA = ma->L;
     k.LB = mb->L;
     k.dR = s.dR;
