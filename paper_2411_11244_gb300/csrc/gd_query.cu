@@ -2091,6 +2091,25 @@ __device__ void leaf_phase(const AT& A, unsigned nleaf, unsigned& tripairs, unsi
 
 // ------------------------------------------------------------- phases 4-6
 
+// The six vertices of a triangle pair in the world frame, on every lane: lanes
+// 0-17 compute one coordinate each, in one path (three float64 instructions in
+// turn, each of which holds the float64 pipe for 64 cycles however many lanes
+// are active; a vertex a lane, A's and B's apart, took eighteen).
+__device__ __forceinline__ void map_pair_warp(const QState& s, const Tri32& TA, const Tri32& TB, V3<double>* Aw,
+                                              V3<double>* Bw) {
+    const int l = min(threadIdx.x & 31u, 17u), k = l / 3, c = l - 3 * k;
+    const double* X = (k < 3 ? s.xa : s.xb) + 4 * c;
+    const double x0 = X[0], x1 = X[1], x2 = X[2], x3 = X[3];
+    const V3<float> v = k < 3 ? pick3(TA.v, k) : pick3(TB.v, k - 3);
+    const double w = fma(x0, (double)v.x, fma(x1, (double)v.y, fma(x2, (double)v.z, x3)));
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        Aw[j] = mk3(__shfl_sync(kFull, w, 3 * j), __shfl_sync(kFull, w, 3 * j + 1), __shfl_sync(kFull, w, 3 * j + 2));
+        Bw[j] = mk3(__shfl_sync(kFull, w, 9 + 3 * j), __shfl_sync(kFull, w, 10 + 3 * j),
+                    __shfl_sync(kFull, w, 11 + 3 * j));
+    }
+}
+
 // float64 distance of one triangle pair in the world frame, computed by a whole
 // warp.  Min kind: lane f owns feature pair f of tri_feature (21 lanes).  A
 // float32 pass on local coordinates first bounds every feature from both
@@ -2107,17 +2126,8 @@ __device__ __noinline__ double refine_pair_warp(const QState& s, unsigned ta, un
     Tri32 TA = load_tri(s.A->tri, ta), TB = load_tri(s.B->tri, tb);
     *ida = TA.id;
     *idb = TB.id;
-    // lanes 0..5 map one vertex each, then share them
-    V3<double> w = mk3(0.0, 0.0, 0.0);
-    if (lane < 3) w = map64(s.xa, (double)TA.v[lane].x, (double)TA.v[lane].y, (double)TA.v[lane].z);
-    else if (lane < 6)
-        w = map64(s.xb, (double)TB.v[lane - 3].x, (double)TB.v[lane - 3].y, (double)TB.v[lane - 3].z);
     V3<double> Aw[3], Bw[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        Aw[k] = mk3(__shfl_sync(kFull, w.x, k), __shfl_sync(kFull, w.y, k), __shfl_sync(kFull, w.z, k));
-        Bw[k] = mk3(__shfl_sync(kFull, w.x, 3 + k), __shfl_sync(kFull, w.y, 3 + k), __shfl_sync(kFull, w.z, 3 + k));
-    }
+    map_pair_warp(s, TA, TB, Aw, Bw);
     V3<double> p = Aw[0], qq = Bw[0];
     double d2 = INFINITY;
     bool hit = false;
@@ -2231,17 +2241,8 @@ __device__ __noinline__ double refine_pair_cta(const QState& s, const float4* tr
     *idb = TB.id;
     __syncthreads();  // the shared results of a previous pair have been read
     if (warp < 3) {
-        V3<double> w = mk3(0.0, 0.0, 0.0);
-        if (lane < 3) w = map64(s.xa, (double)TA.v[lane].x, (double)TA.v[lane].y, (double)TA.v[lane].z);
-        else if (lane < 6)
-            w = map64(s.xb, (double)TB.v[lane - 3].x, (double)TB.v[lane - 3].y, (double)TB.v[lane - 3].z);
         V3<double> Aw[3], Bw[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Aw[k] = mk3(__shfl_sync(kFull, w.x, k), __shfl_sync(kFull, w.y, k), __shfl_sync(kFull, w.z, k));
-            Bw[k] = mk3(__shfl_sync(kFull, w.x, 3 + k), __shfl_sync(kFull, w.y, 3 + k),
-                        __shfl_sync(kFull, w.z, 3 + k));
-        }
+        map_pair_warp(s, TA, TB, Aw, Bw);
         V3<double> p = Aw[0], qq = Bw[0];
         double d2 = INFINITY;
         bool hit = false;
@@ -2326,7 +2327,7 @@ __device__ __noinline__ double refine_pair_cta(const QState& s, const float4* tr
 // candidates are listed for the selection.
 template <int KIND, class AT>
 __device__ void refine_phase_cta(const AT& A, unsigned ncand, unsigned& refined, unsigned long long& bytes) {
-    __shared__ unsigned s_list[kBlock];
+    __shared__ uint4 s_list[kBlock];  // (candidate, ta, tb, query)
     __shared__ unsigned s_n;
     const unsigned long long W = work_ctas(A);
     for (unsigned long long base = blockIdx.x; base < ncand; base += W * blockDim.x) {
@@ -2356,24 +2357,25 @@ __device__ void refine_phase_cta(const AT& A, unsigned ncand, unsigned& refined,
                 keep = KIND == 0 ? (stop ? (st & kStatZero) && c.bound < 0.f : c.bound <= U)
                                  : (!stop && c.bound >= U);
             }
-            if (keep) s_list[atomicAdd(&s_n, 1u)] = (unsigned)i;
+            if (keep) s_list[atomicAdd(&s_n, 1u)] = make_uint4((unsigned)i, c.ta, c.tb, c.q);
             else A.cand_d[i] = __longlong_as_double(-1ll);  // NaN: never selected
         }
         __syncthreads();
         const unsigned n = s_n;
         for (unsigned k = 0; k < n; ++k) {
-            const unsigned ci = s_list[k];
-            float4 raw = __ldcg(reinterpret_cast<const float4*>(A.cand + ci));
-            const Cand c = *reinterpret_cast<Cand*>(&raw);
-            QState& s = A.qs[c.q];
+            const uint4 e = s_list[k];
+            const unsigned ci = e.x;
+            QState& s = A.qs[e.w];
             V3<double> P, Q;
             int ia, ib;
             // (a single query's triangle arrays from the CTA's copy: two
             // dependent loads fewer before the triangles)
             const float4* tA = AT::kOne ? cta().v.triA : s.A->tri;
             const float4* tB = AT::kOne ? cta().v.triB : s.B->tri;
-            const double d = refine_pair_cta<KIND>(s, tA, tB, c.ta, c.tb, &P, &Q, &ia, &ib);
+            const double d = refine_pair_cta<KIND>(s, tA, tB, e.y, e.z, &P, &Q, &ia, &ib);
             if (threadIdx.x == 0) {
+                // (the selection needs the original indices, not the sorted ones)
+                *reinterpret_cast<uint2*>(&A.cand[ci]) = make_uint2((unsigned)ia, (unsigned)ib);
                 double* w = A.cand_pts + 6ull * ci;
                 w[0] = P.x; w[1] = P.y; w[2] = P.z; w[3] = Q.x; w[4] = Q.y; w[5] = Q.z;
                 const unsigned r = atomicAdd(A.ctr + kCtrRefined, 1u);
@@ -2414,9 +2416,7 @@ __device__ void select_phase(const KArgs& A, RefinedSet R, unsigned long long fi
         if (c.q >= (unsigned)A.nq) continue;  // flagged by the refinement
         QState& s = A.qs[c.q];
         if ((unsigned long long)__double_as_longlong(d) == ld_relaxed64(&s.best_d)) {
-            unsigned ia = (unsigned)__float_as_int(__ldg(s.A->tri + 3ull * c.ta + 2).y);
-            unsigned ib = (unsigned)__float_as_int(__ldg(s.B->tri + 3ull * c.tb + 2).y);
-            atomicMin(&s.best_key, ((unsigned long long)ia << 32) | ib);
+            atomicMin(&s.best_key, ((unsigned long long)c.ta << 32) | c.tb);
         }
     }
 }
@@ -2433,61 +2433,35 @@ __device__ void finalize_phase(const KArgs& A, RefinedSet R, unsigned long long 
         if (c.q >= (unsigned)A.nq) continue;  // flagged by the refinement
         QState& s = A.qs[c.q];
         if ((unsigned long long)__double_as_longlong(d) != ld_relaxed64(&s.best_d)) continue;
-        unsigned ia = (unsigned)__float_as_int(__ldg(s.A->tri + 3ull * c.ta + 2).y);
-        unsigned ib = (unsigned)__float_as_int(__ldg(s.B->tri + 3ull * c.tb + 2).y);
-        if ((((unsigned long long)ia << 32) | ib) != ld_relaxed64(&s.best_key)) continue;
+        if ((((unsigned long long)c.ta << 32) | c.tb) != ld_relaxed64(&s.best_key)) continue;
         const double* w = A.cand_pts + 6ull * i;
         gd_result& r = A.out[c.q];
         r.d = d;
-        r.tri_a = ia;
-        r.tri_b = ib;
+        r.tri_a = c.ta;
+        r.tri_b = c.tb;
         r.pa[0] = __ldcg(w); r.pa[1] = __ldcg(w + 1); r.pa[2] = __ldcg(w + 2);
         r.pb[0] = __ldcg(w + 3); r.pb[1] = __ldcg(w + 4); r.pb[2] = __ldcg(w + 5);
     }
 }
 
-// Single query, CTA 0 alone: the witness selection and the result record in
-// one pass (select_phase then finalize_phase load every refined candidate
-// twice, each through a chain of dependent loads): every thread keeps its
-// least original (tri_a, tri_b) at the extreme, the CTA takes the least, and
-// the thread that holds it writes the record.  The triangle arrays come from
-// the CTA's copy of the query's constants.
-__device__ void select_finalize_single(const KArgs& A, RefinedSet R) {
-    __shared__ unsigned long long s_key;
-    if (threadIdx.x == 0) s_key = 0xffffffffffffffffull;
-    __syncthreads();
-    QState& s = A.qs[0];
-    const unsigned long long best = ld_relaxed64(&s.best_d);
-    const float4* triA = cta().v.triA;
-    const float4* triB = cta().v.triB;
-    unsigned long long mykey = 0xffffffffffffffffull;
-    unsigned myi = 0;
-    for (unsigned k = threadIdx.x; k < R.n; k += blockDim.x) {
-        const unsigned i = R.at(k);
-        if (i >= A.cap_cand) continue;
-        if ((unsigned long long)__double_as_longlong(__ldcg(A.cand_d + i)) != best) continue;
-        float4 raw = __ldcg(reinterpret_cast<const float4*>(A.cand + i));
-        const Cand c = *reinterpret_cast<Cand*>(&raw);
-        if (c.q != 0u) continue;  // flagged by the refinement
-        const unsigned ia = (unsigned)__float_as_int(__ldg(triA + 3ull * c.ta + 2).y);
-        const unsigned ib = (unsigned)__float_as_int(__ldg(triB + 3ull * c.tb + 2).y);
-        const unsigned long long key = ((unsigned long long)ia << 32) | ib;
-        if (key < mykey) { mykey = key; myi = i; }
+// The outcome of a query whose status word is st: status and flags of its record,
+// and no distance or pair without GD_OK.
+__device__ __forceinline__ void settle(gd_result& r, unsigned st, double d) {
+    unsigned code = GD_OK;
+    // a proven D_min = 0 stands even if some entries were lost to full
+    // queues or the query was evicted from its batch
+    if (st & kStatEvict) st |= kStatOverflow;
+    if ((st & kStatZero) && !(st & kStatNoResult)) st &= ~kStatOverflow;
+    if (st & kStatOverflow) code = GD_ERR_OVERFLOW;
+    else if (st & kStatTimeout) code = GD_ERR_TIMEOUT;
+    else if (st & kStatNoResult) code = GD_ERR_CUDA;
+    r.status = code;
+    r.flags = (code == GD_OK && d == 0.0) ? 1u : 0u;
+    if (code == GD_OK && (st & kStatZero)) r.flags |= 2u;
+    if (code != GD_OK) {
+        r.d = __longlong_as_double(0x7ff8000000000000ll);
+        r.tri_a = r.tri_b = -1;
     }
-    if (mykey != 0xffffffffffffffffull) atomicMin(&s_key, mykey);
-    __syncthreads();
-    if (mykey != 0xffffffffffffffffull && mykey == s_key) {
-        // ties hold the same pair: equal records
-        const double* w = A.cand_pts + 6ull * myi;
-        gd_result& r = A.out[0];
-        r.d = __longlong_as_double((long long)best);
-        r.tri_a = (long long)(mykey >> 32);
-        r.tri_b = (long long)(mykey & 0xffffffffull);
-        r.pa[0] = __ldcg(w); r.pa[1] = __ldcg(w + 1); r.pa[2] = __ldcg(w + 2);
-        r.pb[0] = __ldcg(w + 3); r.pb[1] = __ldcg(w + 4); r.pb[2] = __ldcg(w + 5);
-        s.best_key = mykey;
-    }
-    __syncthreads();
 }
 
 __device__ void status_phase(const KArgs& A, unsigned long long first, unsigned long long gstride) {
@@ -2495,43 +2469,75 @@ __device__ void status_phase(const KArgs& A, unsigned long long first, unsigned 
         QState& s = A.qs[q];
         unsigned st = ld_relaxed(&s.status);
         if (ld_relaxed64(&s.best_key) == 0xffffffffffffffffull) st |= kStatNoResult;
-        gd_result& r = A.out[q];
-        unsigned code = GD_OK;
-        // a proven D_min = 0 stands even if some entries were lost to full
-        // queues or the query was evicted from its batch
-        if (st & kStatEvict) st |= kStatOverflow;
-        if ((st & kStatZero) && !(st & kStatNoResult)) st &= ~kStatOverflow;
-        if (st & kStatOverflow) code = GD_ERR_OVERFLOW;
-        else if (st & kStatTimeout) code = GD_ERR_TIMEOUT;
-        else if (st & kStatNoResult) code = GD_ERR_CUDA;
-        r.status = code;
-        r.flags = (code == GD_OK && __ldcg(&r.d) == 0.0) ? 1u : 0u;
-        if (code == GD_OK && (st & kStatZero)) r.flags |= 2u;
-        if (code != GD_OK) {
-            r.d = __longlong_as_double(0x7ff8000000000000ll);
-            r.tri_a = r.tri_b = -1;
-        }
+        settle(A.out[q], st, __ldcg(&A.out[q].d));
         if (A.done_ns) A.done_ns[q] = globaltimer();
     }
 }
 
-// A single query's record to the host, by CTA 0 as soon as it is final (every
-// thread calls; the record was written by this CTA before a __syncthreads): the
-// other CTAs' way out and the last one's bookkeeping, about 3 us, are not
-// waited for.  The last CTA out then only stamps HostDone::exit_seq.
-__device__ __forceinline__ void publish_record(const KArgs& A) {
-    if (!A.host_done || A.host_out) return;
-    HostDone* h = A.host_done;
+// Single query, CTA 0 alone: selection, record and its way to the host in one
+// pass.  Every thread keeps its least original (tri_a, tri_b) at the extreme with
+// its points (loads that do not wait for one another), the CTA takes the least,
+// and the thread that holds it makes the record; warp 0 writes that to device
+// memory and, for a synchronous call, to the host: the other CTAs' way out and the
+// last one's bookkeeping, about 3 us, are not waited for (the last CTA out then
+// only stamps HostDone::exit_seq).  One fence orders the record before its stamp.
+template <class AT>
+__device__ void finish_single(const AT& A, RefinedSet R) {
+    __shared__ unsigned long long s_key;
+    __shared__ gd_result s_rec;
     static_assert(sizeof(gd_result) % 8 == 0, "result record copied in 8-byte words");
     constexpr int kW = (int)(sizeof(gd_result) / 8);
-    if (threadIdx.x < kW)
-        reinterpret_cast<unsigned long long*>(&h->out)[threadIdx.x] =
-            __ldcg(reinterpret_cast<const unsigned long long*>(A.out) + threadIdx.x);
-    __threadfence_system();
+    static_assert(kW <= 30, "a lane a word, and two more");
+    if (threadIdx.x == 0) s_key = 0xffffffffffffffffull;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    QState& s = A.qs[0];
+    const unsigned long long best = ld_relaxed64(&s.best_d);
+    const unsigned st = ld_relaxed(&s.status);
+    unsigned long long mykey = 0xffffffffffffffffull;
+    double2 w0 = make_double2(0.0, 0.0), w1 = w0, w2 = w0;
+    for (unsigned k = threadIdx.x; k < R.n; k += blockDim.x) {
+        const unsigned i = R.at(k);
+        if (i >= A.cap_cand) continue;
+        const double d = __ldcg(A.cand_d + i);
+        const uint4 c = __ldcg(reinterpret_cast<const uint4*>(A.cand + i));
+        const double2* w = reinterpret_cast<const double2*>(A.cand_pts + 6ull * i);
+        const double2 p0 = __ldcg(w), p1 = __ldcg(w + 1), p2 = __ldcg(w + 2);
+        if ((unsigned long long)__double_as_longlong(d) != best) continue;
+        const unsigned long long key = ((unsigned long long)c.x << 32) | c.y;
+        if (key < mykey) { mykey = key; w0 = p0; w1 = p1; w2 = p2; }
+    }
+    if (mykey != 0xffffffffffffffffull) atomicMin(&s_key, mykey);
+    __syncthreads();
+    const unsigned long long key = s_key;
+    // ties hold the same pair: equal records
+    if (key != 0xffffffffffffffffull ? mykey == key : threadIdx.x == 0) {
+        gd_result r;
+        r.d = __longlong_as_double((long long)best);
+        r.tri_a = (long long)(key >> 32);
+        r.tri_b = (long long)(key & 0xffffffffull);
+        r.pa[0] = w0.x; r.pa[1] = w0.y; r.pa[2] = w1.x;
+        r.pb[0] = w1.y; r.pb[1] = w2.x; r.pb[2] = w2.y;
+        settle(r, key == 0xffffffffffffffffull ? st | kStatNoResult : st, r.d);
+        s_rec = r;
+        s.best_key = key;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const bool send = A.host_done && !A.host_out;
+    HostDone* h = A.host_done;
+    const int t = threadIdx.x;
+    if (t < kW) {
+        const unsigned long long v = reinterpret_cast<const unsigned long long*>(&s_rec)[t];
+        reinterpret_cast<unsigned long long*>(A.out)[t] = v;
+        if (send) reinterpret_cast<unsigned long long*>(&h->out)[t] = v;
+    } else if (send && t == 30) {
         h->last_abort = 0u;
+    } else if (send && t == 31) {
         h->bad_index = ld_relaxed(A.ctr + kCtrBadIndex);
+    }
+    if (A.done_ns && t == 0) A.done_ns[0] = globaltimer();
+    __syncwarp();
+    if (send && t == 0) {
         __threadfence_system();
         *reinterpret_cast<volatile unsigned long long*>(&h->seq) = A.seq;
         A.ctr[kCtrSent] = 1u;  // (this thread's exit count releases it to the last CTA)
@@ -2891,18 +2897,16 @@ expand:
                     lap(6);
                     const RefinedSet R{nullptr, nc};
                     if (AT::kOne) {
-                        select_finalize_single(A, R);
-                        lap(7);
+                        finish_single(A, R);
                     } else {
                         select_phase(A, R, threadIdx.x, blockDim.x);
                         __syncthreads();
                         lap(7);
                         finalize_phase(A, R, threadIdx.x, blockDim.x);
                         __syncthreads();
+                        status_phase(A, threadIdx.x, blockDim.x);
+                        __syncthreads();
                     }
-                    status_phase(A, threadIdx.x, blockDim.x);
-                    __syncthreads();
-                    if (AT::kOne) publish_record(A);
                     lap(8);
                 }
             }
@@ -2916,11 +2920,7 @@ expand:
             // one query: CTA 0 selects and writes the witness alone (the refined
             // candidates are few), no further grid barrier
             if (blockIdx.x == 0) {
-                select_finalize_single(A, R);
-                lap(7);
-                status_phase(A, threadIdx.x, blockDim.x);
-                __syncthreads();
-                publish_record(A);
+                finish_single(A, R);
                 lap(8);
             }
             goto done;
