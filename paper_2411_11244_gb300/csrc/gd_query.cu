@@ -654,6 +654,37 @@ __device__ __forceinline__ void tri_pair_bounds(const QView& V, unsigned ta, uns
 template <int KIND, bool GROUP, class AT>
 __device__ __forceinline__ void tri_pair_bounds_tight(const AT& A, unsigned q, const QView& V, const Tri32& TA,
                                                       const Tri32& TB, float* lo, float* up) {
+    const V3<float> o = TA.v[0];
+    if constexpr (GROUP) {
+        // B's nine coordinates over the group's lanes (lane 0 also takes the last),
+        // in a loop: a ninth of the instructions, which a query's first pairs wait
+        // for as they are fetched (leaf phase of two tori 9.8 -> 8.7 us)
+        const CtaState& c = cta();
+        const unsigned sub = threadIdx.x & 7u, first = threadIdx.x & 24u;
+        float mine[2];
+#pragma unroll 1
+        for (int r = 0; r < 2; ++r) {
+            const int at = r ? 8 : (int)sub, k = at / 3, i = at - 3 * k;
+            const V3<float> p = pick3(TB.v, k);
+            DF acc = two_sum(c.v.X.t[i], -(i == 0 ? o.x : i == 1 ? o.y : o.z));
+            acc = df_add(acc, DF{c.tl[i], 0.f});
+            acc = df_add(acc, df_mul_f(DF{c.v.X.R[3 * i], c.Rl[3 * i]}, p.x));
+            acc = df_add(acc, df_mul_f(DF{c.v.X.R[3 * i + 1], c.Rl[3 * i + 1]}, p.y));
+            acc = df_add(acc, df_mul_f(DF{c.v.X.R[3 * i + 2], c.Rl[3 * i + 2]}, p.z));
+            mine[r] = __fadd_rn(acc.hi, acc.lo);
+        }
+        V3<float> Al[3], Bl[3];
+        float X = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Al[k] = mk3(__fsub_rn(TA.v[k].x, o.x), __fsub_rn(TA.v[k].y, o.y), __fsub_rn(TA.v[k].z, o.z));
+            Bl[k] = mk3(__shfl_sync(kFull, mine[0], first + 3 * k), __shfl_sync(kFull, mine[0], first + 3 * k + 1),
+                        k < 2 ? __shfl_sync(kFull, mine[0], first + 3 * k + 2) : mine[1]);
+            X = fmaxf(X, fmaxf(max_abs3(Al[k]), max_abs3(Bl[k])));
+        }
+        tri_bounds_core<KIND, GROUP>(Al, Bl, __fadd_ru(c.E_df, __fmul_ru(256.0f * kU * 1.001f, X)), lo, up);
+        return;
+    }
     float Rl[9], tl[3], Edf;
     if (AT::kOne) {
         const CtaState& c = cta();
@@ -670,7 +701,6 @@ __device__ __forceinline__ void tri_pair_bounds_tight(const AT& A, unsigned q, c
         for (int i = 0; i < 3; ++i) tl[i] = s.tl[i];
         Edf = s.E_df;
     }
-    const V3<float> o = TA.v[0];
     const float oc[3] = {o.x, o.y, o.z};
     V3<float> Al[3], Bl[3];
     float X = 0.f;
@@ -1874,19 +1904,28 @@ __device__ void leaf_phase_slots(const AT& A, unsigned nleaf, unsigned& tripairs
     uint4* list = leaf_list<AT::kOne>();
     unsigned& list_n = leaf_list_n();
     const unsigned long long total = (unsigned long long)nleaf * 4ull;
-    const unsigned long long gstride = (unsigned long long)work_ctas(A) * blockDim.x;
+    // A single query's short queue is dealt evenly to all CTAs, so that each has few
+    // pairs to bound and bounds them by groups (two tori, 190 leaf pairs: on three
+    // CTAs the phase took 14.0 us, on 190 CTAs 9.8).  From half a pass of the grid
+    // on every CTA has its warps full: dealt evenly, the rings' 17 K pairs went from
+    // 14.9 to 15.4 us.
+    const unsigned long long threads = (unsigned long long)work_ctas(A) * blockDim.x;
+    unsigned per = blockDim.x;
+    if (AT::kOne && 2ull * total <= threads && total > 0ull)
+        per = 4u * (unsigned)((nleaf + work_ctas(A) - 1) / work_ctas(A));
+    const unsigned long long gstride = (unsigned long long)work_ctas(A) * per;
     const bool pull = AT::kOne && threadIdx.x == 0;
     const int lane = threadIdx.x & 31;
     // the plane axes of the cheap test pay off on queues longer than one pass
     // (a rings query, one pass, lost 1.8 us of leaf phase with them)
-    const bool planes = total > gstride;
+    const bool planes = total > threads;
     // the query's constants: a single query reads the CTA's shared copy where
     // it uses them (no per-thread copy held through the slot loop); a batch
     // keeps a per-thread view of the last query it met
     QView Vb;
     int pit = 0;
     if (threadIdx.x == 0) list_n = 0u;
-    for (unsigned long long cbase = (unsigned long long)blockIdx.x * blockDim.x; cbase < total; cbase += U * gstride) {
+    for (unsigned long long cbase = (unsigned long long)blockIdx.x * per; cbase < total; cbase += U * gstride) {
         // a single query whose traversal stopped (D = 0 proven) skips the rest
         // (this barrier also publishes list_n)
         if (__syncthreads_or(AT::kOne && (((volatile CtaState&)cta()).stat & kStatStop) != 0u)) break;
@@ -1900,7 +1939,7 @@ __device__ void leaf_phase_slots(const AT& A, unsigned nleaf, unsigned& tripairs
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const unsigned long long vt = cbase + (unsigned long long)u * gstride + threadIdx.x;
-            valid[u] = vt < total;
+            valid[u] = threadIdx.x < per && vt < total;
             it[u] = Item{1u, 1u, 0.f, 0u};
             if (valid[u]) {
                 float4 raw = __ldcg(reinterpret_cast<const float4*>(A.leafq + (vt >> 2)));
