@@ -2257,7 +2257,118 @@ __device__ __noinline__ double refine_pair_warp(const QState& s, unsigned ta, un
     return sqrt(-best);
 }
 
-// float64 refinement, one warp per candidate (warps first_warp, +wstride, ...)
+// The features of tri_feature for a warp that gives each three neighbouring lanes,
+// one coordinate a lane (float64, the same operations in the same order, so the
+// same bits).  A float64 instruction holds its SM sub-partition's pipe for 64
+// cycles however many lanes are active, so a lane per feature spent about 130 of
+// them in turn on an edge pair; three lanes per feature take about 70.
+struct Lane3 {
+    int base, c, c1, c2;  // the feature's first lane, this lane's coordinate and the next two
+    __device__ __forceinline__ double get(double x, int k) const { return __shfl_sync(kFull, x, base + k); }
+    __device__ __forceinline__ double cross(double a, double b) const {
+        return ssub(smul(get(a, c1), get(b, c2)), smul(get(a, c2), get(b, c1)));
+    }
+    __device__ __forceinline__ double dot(double a, double b) const {
+        const double m = smul(a, b);
+        return sadd(sadd(get(m, 0), get(m, 1)), get(m, 2));
+    }
+    // three dot products from their coordinates' products, one summed by each lane
+    __device__ __forceinline__ void sums(double m0, double m1, double m2, double* r0, double* r1, double* r2) const {
+        double x[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double g0 = get(m0, k), g1 = get(m1, k), g2 = get(m2, k);
+            x[k] = c == 0 ? g0 : (c == 1 ? g1 : g2);
+        }
+        const double t = sadd(sadd(x[0], x[1]), x[2]);
+        *r0 = get(t, 0);
+        *r1 = get(t, 1);
+        *r2 = get(t, 2);
+    }
+    __device__ __forceinline__ double of(V3<double> v) const { return c == 0 ? v.x : (c == 1 ? v.y : v.z); }
+};
+
+// Edge pair (i, j): closest_segment_segment with its coordinates on three lanes.
+__device__ __forceinline__ void edges_lane3(const Lane3& L, int i, int j, const V3<double>* A, const V3<double>* B,
+                                            double* P, double* Q, double* dist2) {
+    const double p0 = L.of(pick3(A, i)), q0 = L.of(pick3(B, j));
+    const double d1 = ssub(L.of(pick3(A, i == 2 ? 0 : i + 1)), p0);
+    const double d2 = ssub(L.of(pick3(B, j == 2 ? 0 : j + 1)), q0);
+    const double r = ssub(p0, q0);
+    double a, e, f, c, b, den, num, unused;
+    L.sums(smul(d1, d1), smul(d2, d2), smul(d2, r), &a, &e, &f);
+    const double n = L.cross(d1, d2), m = L.cross(d2, r);
+    const double cr = smul(d1, r), bd = smul(d1, d2);
+    L.sums(cr, bd, smul(n, n), &c, &b, &den);
+    L.sums(smul(n, m), cr, bd, &num, &unused, &unused);
+    double s, t;
+    if (!(a > 0.0)) {
+        s = 0.0;
+        t = e > 0.0 ? clamp_div(f, e) : 0.0;
+    } else if (!(e > 0.0)) {
+        t = 0.0;
+        s = clamp_div(-c, a);
+    } else {
+        s = den > 0.0 ? clamp_div(num, den) : 0.0;
+        const double tn = sadd(smul(b, s), f);
+        const bool lo = tn < 0.0, hi = tn > e;
+        const double u = clamp_div(lo ? -c : (hi ? ssub(b, c) : tn), (lo || hi) ? a : e);
+        t = lo ? 0.0 : (hi ? 1.0 : u);
+        if (lo || hi) s = u;
+    }
+    *P = sadd(p0, smul(d1, s));
+    *Q = sadd(q0, smul(d2, t));
+    const double d = ssub(*P, *Q);
+    *dist2 = L.dot(d, d);
+}
+
+// Vertex k of A against B (va) or of B against A: project_into_triangle.
+__device__ __forceinline__ void vertex_lane3(const Lane3& L, bool va, int k, const V3<double>* A, const V3<double>* B,
+                                             double* P, double* Q, double* dist2) {
+    const double v = L.of(va ? pick3(A, k) : pick3(B, k));
+    const double t0 = L.of(va ? B[0] : A[0]);
+    const double e0 = ssub(L.of(va ? B[1] : A[1]), t0), e1 = ssub(L.of(va ? B[2] : A[2]), t0), w = ssub(v, t0);
+    const double n = L.cross(e0, e1), u = L.cross(w, e1), z = L.cross(e0, w);
+    double det, un, vn;
+    L.sums(smul(n, n), smul(u, n), smul(z, n), &det, &un, &vn);
+    const bool in = det > 0.0 && un >= 0.0 && vn >= 0.0 && sadd(un, vn) <= det;
+    if (!__any_sync(kFull, in)) return;
+    const double g = in ? sdiv(L.c == 1 ? vn : un, det) : 0.0;
+    const double c = sadd(sadd(t0, smul(e0, L.get(g, 0))), smul(e1, L.get(g, 1)));
+    const double p = va ? v : c, q = va ? c : v, d = ssub(p, q);
+    const double dd = L.dot(d, d);
+    if (in) {
+        *P = p;
+        *Q = q;
+        *dist2 = dd;
+    }
+}
+
+// Edge k of A crossing B's plane (ea) or of B crossing A's, inside the triangle: a hit.
+__device__ __forceinline__ void plane_lane3(const Lane3& L, bool ea, int k, const V3<double>* A, const V3<double>* B,
+                                            double* P, double* Q, double* dist2, bool* hit) {
+    const int j = k == 2 ? 0 : k + 1;
+    const double e0 = L.of(ea ? pick3(A, k) : pick3(B, k)), e1 = L.of(ea ? pick3(A, j) : pick3(B, j));
+    const double f0 = L.of(ea ? B[0] : A[0]);
+    const double fa = ssub(L.of(ea ? B[1] : A[1]), f0), fb = ssub(L.of(ea ? B[2] : A[2]), f0);
+    const double n = L.cross(fa, fb);
+    const double nn = smul(n, n);
+    double si, sj, det, un, vn, unused;
+    L.sums(smul(n, ssub(e0, f0)), smul(n, ssub(e1, f0)), nn, &si, &sj, &det);
+    const double den = ssub(si, sj);
+    const bool crosses = ((si <= 0.0 && sj >= 0.0) || (si >= 0.0 && sj <= 0.0)) && den != 0.0;
+    if (!__any_sync(kFull, crosses)) return;
+    const double X = sadd(e0, smul(ssub(e1, e0), crosses ? clamp01(sdiv(si, den)) : 0.0));
+    const double w = ssub(X, f0);
+    L.sums(smul(L.cross(w, fb), n), smul(L.cross(fa, w), n), nn, &un, &vn, &unused);
+    if (crosses && det > 0.0 && un >= 0.0 && vn >= 0.0 && sadd(un, vn) <= det) {
+        *hit = true;
+        *P = X;
+        *Q = X;
+        *dist2 = 0.0;
+    }
+}
+
 // float64 distance of one triangle pair computed by three warps of a CTA, one
 // per kind of feature pair: warp 0 the 9 edge-edge pairs, warp 1 the 6
 // vertex-face pairs, warp 2 the 6 edge-plane crossings (max kind: warp 0, the
@@ -2282,21 +2393,25 @@ __device__ __noinline__ double refine_pair_cta(const QState& s, const float4* tr
     if (warp < 3) {
         V3<double> Aw[3], Bw[3];
         map_pair_warp(s, TA, TB, Aw, Bw);
-        V3<double> p = Aw[0], qq = Bw[0];
+        // three lanes a feature (min) or vertex pair (max), a coordinate each; the
+        // lanes left over repeat the last one, and of equal values the first
+        // lane wins, which is a first coordinate's
+        const int g = min(lane / 3, warp == 0 ? 8 : 5), c = lane % 3;
+        const Lane3 L{3 * g, c, c == 2 ? 0 : c + 1, c == 0 ? 2 : c - 1};
+        const int gi = g / 3, gj = g - 3 * gi;
+        double p = L.of(Aw[0]), qq = L.of(Bw[0]);
         double d2 = INFINITY;
         bool hit = false;
-        int f = 99;
+        const int f = g + (warp == 0 ? 0 : (warp == 1 ? 9 : 15));
         if (KIND == 0) {
-            const bool on = warp == 0 ? lane < 9 : lane < 6;
-            f = warp == 0 ? lane : (warp == 1 ? 9 + lane : 15 + lane);
-            if (on) tri_feature(f, Aw, Bw, &p, &qq, &d2, &hit);
-            else f = 99;
-        } else if (warp == 0 && lane < 9) {
-            p = Aw[lane / 3];
-            qq = Bw[lane % 3];
-            const V3<double> d = p - qq;
-            d2 = -dot(d, d);  // reduce with min
-            f = lane;
+            if (warp == 0) edges_lane3(L, gi, gj, Aw, Bw, &p, &qq, &d2);
+            else if (warp == 1) vertex_lane3(L, gi == 0, gj, Aw, Bw, &p, &qq, &d2);
+            else plane_lane3(L, gi == 0, gj, Aw, Bw, &p, &qq, &d2, &hit);
+        } else if (warp == 0) {
+            p = L.of(pick3(Aw, gi));
+            qq = L.of(pick3(Bw, gj));
+            const double d = ssub(p, qq);
+            d2 = -L.dot(d, d);  // reduce with min
         }
         const unsigned hits = __ballot_sync(kFull, hit);
         double best;
@@ -2327,9 +2442,9 @@ __device__ __noinline__ double refine_pair_cta(const QState& s, const float4* tr
                 if (ob < best || (ob == best && ow < win)) { best = ob; win = ow; }
             }
         }
-        const double px = __shfl_sync(kFull, p.x, win), py = __shfl_sync(kFull, p.y, win),
-                     pz = __shfl_sync(kFull, p.z, win), qx = __shfl_sync(kFull, qq.x, win),
-                     qy = __shfl_sync(kFull, qq.y, win), qz = __shfl_sync(kFull, qq.z, win);
+        const double px = __shfl_sync(kFull, p, win), py = __shfl_sync(kFull, p, win + 1),
+                     pz = __shfl_sync(kFull, p, win + 2), qx = __shfl_sync(kFull, qq, win),
+                     qy = __shfl_sync(kFull, qq, win + 1), qz = __shfl_sync(kFull, qq, win + 2);
         const int fw = __shfl_sync(kFull, f, win);
         if (lane == 0) {
             s_d2[warp] = (KIND == 0 && hits) ? -1.0 : best;
