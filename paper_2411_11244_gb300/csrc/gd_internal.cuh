@@ -66,7 +66,7 @@ struct __align__(16) QPack {
     const float* boxB;
     unsigned slot_base;
     unsigned TA, TB;              // triangles
-    unsigned pad;
+    float E_tri;
     const float4* triA;
     const float4* triB;
     float R[9], t[3];             // B-local -> A-local, float32

@@ -212,6 +212,8 @@ __device__ __forceinline__ Rigid32 map_of(const QPack* k) {
     return Rigid32{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x}, {c.y, c.z, c.w}};
 }
 __device__ __forceinline__ Rigid32 map_of(const BView& V) { return map_of(V.k); }
+__device__ __forceinline__ float tri_widening(const QView& V) { return V.E_tri; }
+__device__ __forceinline__ float tri_widening(const BView& V) { return V.k->E_tri; }
 
 // Per-CTA shared copies of global state, refreshed by thread 0 right after
 // every grid barrier (the barrier's closing __syncthreads publishes them):
@@ -805,57 +807,143 @@ __device__ __forceinline__ bool tri_pair_may_hold(const QConst& V, const Tri32& 
 
 // ------------------------------------------------------------- pair bounds
 
+// A node pair along the line d between its boxes' centres (B's box, mapped by X
+// unless AA, as it lies: turned against the axes).
+struct CentreLine {
+    float dd;      // |d|^2
+    float ra, rb;  // extents of the two boxes along d, times |d|
+    float ma, mb;  // the largest of each one's three terms
+    float ha, hb;  // squared half-diagonals
+    float mm;      // product of the largest half-extents
+};
+
+template <bool AA>
+__device__ __forceinline__ CentreLine centre_line(const Rigid32& X, const Box& a, const Box& b) {
+    float h[3], m[3], ha[3], d[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        m[k] = 0.5f * (b.lo[k] + b.hi[k]);
+        h[k] = 0.5f * (b.hi[k] - b.lo[k]);
+        ha[k] = 0.5f * (a.hi[k] - a.lo[k]);
+    }
+    CentreLine c;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float w =
+            AA ? m[k] : fmaf(X.R[3 * k], m[0], fmaf(X.R[3 * k + 1], m[1], fmaf(X.R[3 * k + 2], m[2], X.t[k])));
+        d[k] = w - 0.5f * (a.lo[k] + a.hi[k]);
+    }
+    float ta[3], tb[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float g = AA ? d[k] : fmaf(X.R[k], d[0], fmaf(X.R[3 + k], d[1], X.R[6 + k] * d[2]));
+        ta[k] = fabsf(d[k]) * ha[k];
+        tb[k] = fabsf(g) * h[k];
+    }
+    c.dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
+    c.ra = ta[0] + ta[1] + ta[2];
+    c.rb = tb[0] + tb[1] + tb[2];
+    c.ma = fmaxf(ta[0], fmaxf(ta[1], ta[2]));
+    c.mb = fmaxf(tb[0], fmaxf(tb[1], tb[2]));
+    c.ha = fmaf(ha[0], ha[0], fmaf(ha[1], ha[1], ha[2] * ha[2]));
+    c.hb = fmaf(h[0], h[0], fmaf(h[1], h[1], h[2] * h[2]));
+    c.mm = fmaxf(ha[0], fmaxf(ha[1], ha[2])) * fmaxf(h[0], fmaxf(h[1], h[2]));
+    return c;
+}
+
+// Whether Eq. 10 (Eq. 11) of the pair may improve the running bound U.  Faces i and
+// j have centres c_i, c_j at |c_i - c_j|^2 >= dd + a_i^2 + b_j^2 - 2 (ma + mb + mm)
+// (a_i, b_j: their boxes' half-extents across them), and some pair of their
+// corners is as far apart as |c_i - c_j|^2 plus both squared half-diagonals, so
+// Eq. 10 is at least dd + ha + hb - 2 (ma + mb + mm).  Eq. 11 does not exceed a
+// distance of two face centres.  (An update left out only costs bound.)
+template <int KIND>
+__device__ __forceinline__ bool may_improve(const CentreLine& c, float U) {
+    const float x = 2.f * (c.ma + c.mb + c.mm);
+    if (KIND == 0) return !(c.dd + c.ha + c.hb - x > U * U);
+    return !(c.dd + c.ha + c.hb + x < U * U);
+}
+
+// Whether the boxes' extents along d rule the pair out.  Min: their gap along d is
+// a lower bound of the distance, tighter than the gap between A's box and the
+// box around B's turned one (which is up to sqrt(3) times its size).  Max: |d + w|^2
+// <= |d|^2 + 2 (ra + rb) + (half-diagonals)^2.  The float32 errors (map, centres,
+// extents and the sums) stay below 120 u times the scene's largest coordinate,
+// 256 u of which are in E_tri.
+template <int KIND>
+__device__ __forceinline__ bool line_apart(const CentreLine& c, float U, float E_tri) {
+    if (KIND == 0) {
+        const float num = c.dd - c.ra - c.rb;
+        return num > 0.f && lower_from_dist(num / sqrtf(c.dd), E_tri) > U;
+    }
+    const float s2 = c.dd + 2.f * (c.ra + c.rb) + (c.ha + c.hb + 2.f * sqrtf(c.ha * c.hb));
+    return upper_from_sq(s2, E_tri) < U;
+}
+
 // Bounds of node pair (ia of A, ib of B at depth db).  Returns the stored
 // culling value (KIND 0: squared lower bound of the min; KIND 1: squared upper
 // bound of the max) and whether the pair survives against Ucur; for a
 // survivor, *newU is its enhanced bound (Eq. 10 / Eq. 11) for the running
 // bound and *key orders survivors by it.
 // slot: B's refit slot (refit_slot), looked up by the caller.
-template <int KIND, bool FULL, class VT>
+// LINE: survivors are also tested along their centre line, and the enhanced bound,
+// six times the work of the rest, is evaluated only where it may improve the
+// running bound (*newU and *key are left as they are otherwise): 256 gear queries
+// 16.3 -> 14.0 ms.  TURN: with a refit box of B too, B's own box is tested along
+// that line; a flat patch that lies along B's axes is thin in that box and thick in
+// the refit one (leaf pairs of the gear batch 165 M -> 39 M, 14.0 -> 7.5 ms).
+template <int KIND, bool FULL, bool LINE, bool TURN, class VT>
 __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
                                                 unsigned slot, float Ucur, bool* survive, unsigned* newU,
                                                 unsigned* key) {
-    Box ba = load_box(V.boxA, ia);
+    Box ba = load_box(V.boxA, ia), b0;
+    if (TURN) b0 = load_box(V.boxB, ib);  // (before the refit box is waited for)
     float bound;
     *key = 0xffffffffu;
     if (slot != kNoSlot) {
         // B's box already in A's frame (refit): plain AABB-AABB bounds (no map)
         const Rigid32 none{};
         Box bb = FULL ? load_box_cg(A.ftree, ib) : load_box_cg(A.rbox, refit_index(V, slot, ib, db));
-        if (KIND == 0) {
-            bound = lower_min_sq(ba, bb.lo, bb.hi);
-            *survive = bound <= min_keep_threshold(Ucur, V.E_box);
-            if (*survive) {
+        bound = KIND == 0 ? lower_min_sq(ba, bb.lo, bb.hi) : upper_max_sq(ba, bb.lo, bb.hi);
+        *survive = KIND == 0 ? bound <= min_keep_threshold(Ucur, V.E_box) : bound >= max_keep_threshold(Ucur, V.E_box);
+        if (LINE) {
+            if (!*survive) return bound;
+            if (TURN && line_apart<KIND>(centre_line<false>(map_of(V), ba, b0), Ucur, tri_widening(V))) {
+                *survive = false;
+                return bound;
+            }
+            if (!may_improve<KIND>(centre_line<true>(none, ba, bb), Ucur)) return bound;
+        }
+        if (*survive) {
+            if (KIND == 0) {
                 float u2 = A.conventional ? upper_max_sq(ba, bb.lo, bb.hi) : upper_min_sq_enhanced<true>(none, ba, bb);
                 *newU = __float_as_uint(upper_from_sq(u2, V.E_box));
                 *key = __float_as_uint(u2);
-            }
-        } else {
-            bound = upper_max_sq(ba, bb.lo, bb.hi);
-            *survive = bound >= max_keep_threshold(Ucur, V.E_box);
-            if (*survive) {
+            } else {
                 float l2 = A.conventional ? lower_min_sq(ba, bb.lo, bb.hi) : lower_max_sq_enhanced<true>(none, ba, bb);
                 *newU = __float_as_uint(lower_from_sq(l2, V.E_box));
                 *key = ~__float_as_uint(l2);
             }
         }
     } else {
-        Box bb = load_box(V.boxB, ib);
+        const Box bb = TURN ? b0 : load_box(V.boxB, ib);
         const Rigid32& X = map_of(V);
         float elo[3], ehi[3];
         enclose(X, bb, elo, ehi);
-        if (KIND == 0) {
-            bound = lower_min_sq(ba, elo, ehi);
-            *survive = bound <= min_keep_threshold(Ucur, V.E_box);
-            if (*survive) {
+        bound = KIND == 0 ? lower_min_sq(ba, elo, ehi) : upper_max_sq(ba, elo, ehi);
+        *survive = KIND == 0 ? bound <= min_keep_threshold(Ucur, V.E_box) : bound >= max_keep_threshold(Ucur, V.E_box);
+        if (LINE) {
+            if (!*survive) return bound;
+            const CentreLine c = centre_line<false>(X, ba, bb);
+            if (line_apart<KIND>(c, Ucur, tri_widening(V))) *survive = false;
+            if (!*survive || !may_improve<KIND>(c, Ucur)) return bound;
+        }
+        if (*survive) {
+            if (KIND == 0) {
                 float u2 = A.conventional ? upper_max_sq(ba, elo, ehi) : upper_min_sq_enhanced<false>(X, ba, bb);
                 *newU = __float_as_uint(upper_from_sq(u2, V.E_box));
                 *key = __float_as_uint(u2);
-            }
-        } else {
-            bound = upper_max_sq(ba, elo, ehi);
-            *survive = bound >= max_keep_threshold(Ucur, V.E_box);
-            if (*survive) {
+            } else {
                 float l2 = A.conventional ? lower_min_sq(ba, elo, ehi) : lower_max_sq_enhanced<false>(X, ba, bb);
                 *newU = __float_as_uint(lower_from_sq(l2, V.E_box));
                 *key = ~__float_as_uint(l2);
@@ -865,11 +953,11 @@ __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, uns
     return bound;
 }
 
-template <int KIND, bool FULL = false, class VT>
+template <int KIND, bool FULL = false, bool LINE = false, bool TURN = false, class VT>
 __device__ __forceinline__ float pair_bounds(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
                                              float Ucur, bool* survive, unsigned* newU, unsigned* key) {
     // FULL: B's whole tree was refit into A's frame at the start of the launch
-    return pair_bounds_at<KIND, FULL>(A, V, ia, ib, db, FULL ? 0u : refit_slot(A, V, ib, db), Ucur, survive, newU, key);
+    return pair_bounds_at<KIND, FULL, LINE, TURN>(A, V, ia, ib, db, FULL ? 0u : refit_slot(A, V, ib, db), Ucur, survive, newU, key);
 }
 
 // ------------------------------------------------------------- refit
@@ -1408,6 +1496,7 @@ __device__ void setup_query(const KArgs& A, int q, int kind) {
     setup_state(s, kind, slot_base, mb->L, A.refit);
     QPack& k = s.pk;
     k.E_box = E.E_box;
+    k.E_tri = E.E_tri;
     k.LA = ma->L;
     k.LB = mb->L;
     k.dR = s.dR;
@@ -1562,9 +1651,12 @@ __device__ void expand_level(const AT& A, int level, unsigned n, int s, unsigned
         unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key;
         if (valid) {
             ++pairs;
-            bound = pair_bounds<KIND, FULL>(A, V, ia, ib, dBc, Ucur, &survive, &newU, &key);
+            // (not for a single min query: its levels here are short, and the line
+            // test's instructions cost the rings and spheres 0.5-0.8 us a level)
+            constexpr bool kLine = KIND == 1 || !AT::kOne;
+            bound = pair_bounds<KIND, FULL, kLine, kLine && KIND == 0>(A, V, ia, ib, dBc, Ucur, &survive, &newU, &key);
         }
-        warp_bound_update<KIND>(A, survive, q, newU);
+        warp_bound_update<KIND>(A, survive && newU != (KIND == 0 ? 0xffffffffu : 0u), q, newU);
         if (A.q_budget) {
             // a batch query that pushes more than its share of the queues in
             // this level takes the excess from the launch's common pool; when
@@ -1605,8 +1697,7 @@ __device__ void expand_level(const AT& A, int level, unsigned n, int s, unsigned
     }
 }
 
-// A batch level of one tree level each (s = 2) whose front outgrows the
-// grid: one thread per front entry and its (up to) four child pairs, so that
+// A level of one tree level each (s = 2) with a front that fills the grid: one thread per front entry and its (up to) four child pairs, so that
 // the entry's load, its query's view and running bound, and the warp's
 // collective steps (bound update, queue shares, CTA append) run once per
 // entry instead of once per child pair.  Same bounds, survivors and queue
@@ -1682,14 +1773,14 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
                 bool survive = false;
                 unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key;
                 if (!one_root) slot = refit_slot(A, V, ib, dBc);
-                o[c].bound = pair_bounds_at<KIND, false>(A, V, ia, ib, dBc, slot, Ucur, &survive, &newU, &key);
+                o[c].bound = pair_bounds_at<KIND, false, true, KIND == 0>(A, V, ia, ib, dBc, slot, Ucur, &survive, &newU, &key);
                 if (survive) {
                     sm |= 1u << c;
                     best = KIND == 0 ? min(best, newU) : max(best, newU);
                 }
             }
         }
-        warp_bound_update<KIND>(A, sm != 0u, q, best);
+        warp_bound_update<KIND>(A, best != (KIND == 0 ? 0xffffffffu : 0u), q, best);
         if (A.q_budget) {
             // the queue shares (as in expand_level), one atomic per query
             // among the warp's lanes with survivors
@@ -1740,10 +1831,7 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
 }
 
 // A single query's copy of it, out of line so that the level loop keeps its
-// registers; taken where the front outgrows the grid: from twice its threads on
-// for the min (gears 194 -> 189 us, spheres apart 182 -> 178), from six times for
-// the max (8.9 M entries: 9.07 -> 8.39 ms, but icospheres, 303,000, 188 -> 190 us
-// with the min's rule).
+// registers.
 template <int KIND, class AT>
 __device__ __noinline__ void expand_entries_single(const AT& A, int level, unsigned n, unsigned long long& pairs,
                                                    unsigned long long& bytes) {
@@ -2971,11 +3059,14 @@ expand:
         }
         if (A.q_budget)  // the counters of this level's pushes are those of level + 2
             for (int q = (int)gfirst; q < A.nq; q += (int)gstride) A.qs[q].pushed[level & 1] = 0u;
-        // a batch front of more than twice the grid's threads at one tree
-        // level each: a thread per entry
-        if (!AT::kOne && s == 2 && (unsigned long long)n > 2ull * gstride)
+        // fronts at one tree level each: a thread per entry, in a batch from as
+        // many entries as the grid has threads (256 gears: from twice as many 7.45
+        // ms, as many 7.4, half 7.4), in a single query from half as many
+        // (icosphere max calls: six times 184 us, twice 179, as many 172.4, half 171.6;
+        // torus min: twice 137, as many 131, half 130)
+        if (!AT::kOne && s == 2 && (unsigned long long)n > gstride)
             expand_level_entries<KIND>(A, level, n, pairs, bytes);
-        else if (AT::kOne && !FULL && s == 2 && (unsigned long long)n > (KIND == 0 ? 2ull : 6ull) * gstride)
+        else if (AT::kOne && !FULL && s == 2 && 2ull * n > gstride)
             expand_entries_single<KIND>(A, level, n, pairs, bytes);
         else
             expand_level<KIND, FULL>(A, level, n, s, pairs, bytes);

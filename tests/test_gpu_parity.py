@@ -368,6 +368,24 @@ def test_batch_eviction_matches_single(G, oracle_mod):
         G.gd_ctx_destroy(c)
 
 
+@pytest.mark.parametrize("ta,tb", [(1, 1), (1, 40), (2, 3), (7, 200), (33, 31), (64, 65), (130, 1), (300, 257)])
+def test_small_pairs_of_uneven_depth(G, ctx, oracle_mod, ta, tb):
+    """The first level of a plain call over trees that end within it on one side or
+    both, and leaf queues from one pair to a few hundred (dealt to the CTAs,
+    bounded by groups of lanes): plain calls and a batch against every pair."""
+    rng = np.random.default_rng(31 * ta + tb)
+    A, B = _soup(rng, ta), _soup(rng, tb)
+    xf = [(_rigid(rng, 0.5), _rigid(rng, s)) for s in (0.2, 3.0, 40.0)]
+    run_pair(G, ctx, oracle_mod, A, B, xf)
+    ma, mb = _mesh(G, ctx, A), _mesh(G, ctx, B)
+    items = [(ma, mb, xa, xb, k) for xa, xb in xf for k in (G.GD_MIN, G.GD_MAX)]
+    for r, (_, _, xa, xb, k) in zip(G.gd_batch_query(ctx, items), items):
+        fn = G.gd_min_distance if k == G.GD_MIN else G.gd_max_distance
+        same_answer(r, fn(ctx, ma, mb, xa, xb), oracle_mod, A, xa, B, xb, "min" if k == G.GD_MIN else "max")
+    for h in (ma, mb):
+        G.gd_mesh_destroy(h)
+
+
 def test_refit_modes_agree(G, oracle_mod):
     """Refitting B only tightens bounds: with the lazy refit of B's low
     subtrees (mode 1), without refit (mode 2) and with the paper's full refit
@@ -1224,6 +1242,60 @@ def test_gears_batch_forms_and_plain_calls(G, ctx, oracle_mod):
                 if kind == "min":
                     check(out[i], A, xa, B, xbs[i], kind, refs[k], diag, oracle_mod)
                 check(fn(ctx, ma, mb, xa, xbs[i]), A, xa, B, xbs[i], kind, refs[k], diag, oracle_mod)
+    finally:
+        G.gd_mesh_destroy(ma)
+        G.gd_mesh_destroy(mb)
+
+
+def _plate(n, at):
+    """A square plate of 2 n^2 triangles in the plane z = at of its own frame, centred at (at, at, at)."""
+    g = np.linspace(-1.0, 1.0, n + 1)
+    x, y = np.meshgrid(g, g, indexing="ij")
+    v = (np.stack([x.ravel(), y.ravel(), np.zeros(x.size)], 1) + at).astype(np.float32)
+    k = (np.arange(n)[:, None] * (n + 1) + np.arange(n)[None, :]).ravel()
+    t = np.concatenate([np.stack([k, k + n + 1, k + 1], 1), np.stack([k + 1, k + n + 1, k + n + 2], 1)])
+    return v, t.astype(np.int32)
+
+
+@pytest.mark.parametrize("at", [0.0, 50.0, 1e4])
+@pytest.mark.parametrize("n", [3, 17, 48])
+def test_turned_flat_patches(G, ctx, oracle_mod, n, at):
+    """Flat patches turned against the axes of both frames, where a pair's test
+    along its centre line and the refit box disagree most, nearly parallel and
+    tilted, near their frame's origin and far from it (where the float32
+    errors that the test allows for are largest): plain calls and one batch, both kinds."""
+    rng = np.random.default_rng(1000 * n + int(at))
+    A, B = _plate(n, at), _plate(n + 1, at)
+    c = np.full(3, at)
+    # float64 rounding of the world coordinates, which the translation takes back to
+    # the origin: per coordinate 4 u of at most 2 sqrt(3) (at + 1), over three
+    # coordinates of two points and two evaluations 97 u (at + 1)
+    tol = 128 * 2.0 ** -53 * (at + 1.0)
+    ma, mb = _mesh(G, ctx, A), _mesh(G, ctx, B)
+    try:
+        items = []
+        for i, tilt in enumerate([0.0, 1e-4, 0.03, 0.7]):
+            R, S = synth.random_rotation(rng), synth.random_rotation(rng)
+            ax = rng.normal(size=3)
+            ax *= tilt / np.linalg.norm(ax)
+            K = np.array([[0, -ax[2], ax[1]], [ax[2], 0, -ax[0]], [-ax[1], ax[0], 0]])
+            W = np.linalg.qr(np.eye(3) + K)[0]
+            W *= np.sign(np.diag(W))[None, :]
+            Rb = R @ W
+            xa = synth.xform(R, -R @ c)
+            xb = synth.xform(Rb, -Rb @ c + R[:, 2] * (0.3 + 1.2 * (tilt > 0.5)))
+            items += [(ma, mb, xa, xb, k) for k in (G.GD_MIN, G.GD_MAX)]
+        out = G.gd_batch_query(ctx, items)
+        for r, (_, _, xa, xb, k) in zip(out, items):
+            kind = "min" if k == G.GD_MIN else "max"
+            ref = oracle_mod.brute(A, xa, B, xb, kind) if n < 17 else None
+            if ref is None:
+                ref = oracle_mod.bvh_query(oracle_mod.Bvh(A), xa, oracle_mod.Bvh(B), xb, kind)
+            one = (G.gd_min_distance if kind == "min" else G.gd_max_distance)(ctx, ma, mb, xa, xb)
+            assert one.status == 0 and abs(one.d - ref.d) <= tol, (kind, one.d, ref.d)
+            dw, _, _ = oracle_mod.witness_distance(A, xa, B, xb, one.tri_a, one.tri_b, kind)
+            assert abs(dw - one.d) <= tol, (kind, dw, one.d)
+            same_answer(r, one, oracle_mod, A, xa, B, xb, kind)
     finally:
         G.gd_mesh_destroy(ma)
         G.gd_mesh_destroy(mb)
