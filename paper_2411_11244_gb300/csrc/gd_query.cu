@@ -1697,10 +1697,11 @@ __device__ void expand_level(const AT& A, int level, unsigned n, int s, unsigned
     }
 }
 
-// A level of one tree level each (s = 2) with a front that fills the grid: one thread per front entry and its (up to) four child pairs, so that
-// the entry's load, its query's view and running bound, and the warp's
-// collective steps (bound update, queue shares, CTA append) run once per
-// entry instead of once per child pair.  Same bounds, survivors and queue
+// A level of one tree level each (s = 2) with a front that fills the grid: one
+// thread per front entry and its (up to) four child pairs, so that the entry's
+// load, its query's view and running bound, and the warp's collective steps
+// (bound update, queue shares, CTA append) run once per entry instead of once
+// per child pair.  Same bounds, survivors and queue
 // contents (up to order) as expand_level.
 template <int KIND, class AT>
 __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigned long long& pairs,
@@ -2823,9 +2824,8 @@ __device__ bool refit_jobs(const AT& A, bool lead, unsigned& refits, bool* ran) 
 // query (nq == 1) or a batch; with the query count known at compile time
 // every single-query / batch branch of the inlined phases folds, so each
 // instantiation carries only its own code and register pressure.
-// CTAs per SM of a batch: 3 (80 registers) once its levels and leaf phase load a
-// query's constants per entry (256 gear queries: 17.5 ms; 4 CTAs 18.1, and
-// 20.7 with the constants kept in registers, which then lived in local memory).
+// CTAs per SM of a batch: 3 (80 registers), as its levels and leaf phase load a
+// query's constants per entry (256 gear queries: 6.6 ms; 2 CTAs 7.5, 4 CTAs 7.2).
 #ifndef GD_BATCH_CTAS
 #define GD_BATCH_CTAS 3
 #endif
