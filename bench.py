@@ -331,17 +331,18 @@ def build_roofline(G, meshes, peak, peak_kind):
     """BVH build (Section 7.3 preprocessing) against the HBM roofline: device
     time of the build's kernels (gd_mesh_build_time) and the bytes the build
     must move per triangle T, vertex V and node N: index validation (12 B/T +
-    12 B/V read), Morton codes (12 B/T + 12 B/V read, 12 B/T of key and value
-    written), 8 radix passes of 8 bits over the 63-bit codes (8 B/T histogram
-    read, 12 B/T read and 12 B/T written by the scatter: 256 B/T), the sorted
-    order copied (8 B/T), leaves (4 B/T order + 12 B/T indices + 12 B/V read,
+    12 B/V read), Morton codes (12 B/T + 12 B/V read, 8 B/T of key written), the
+    radix passes that the triangle count calls for (12 B/T read and 12 B/T
+    written each; the first reads no values), the order within equal keys (12 B/T
+    read, 4 B/T written), leaves (4 B/T order + 12 B/T indices + 12 B/V read,
     48 B/T triangle records and 12 B/T vertex indices in leaf order, for the
     refits, written) and 24 B per node box written."""
     out = []
     for h, T, V in meshes:
         L, _ = G.gd_mesh_info(h)
         ms = G.gd_mesh_build_time(h)
-        alg = 376 * T + 36 * V + 24 * ((2 << L) - 1)
+        passes = min(8, max(2, (3 * T.bit_length() // 2 + 6) // 8))
+        alg = (120 + 24 * passes) * T + 36 * V + 24 * ((2 << L) - 1)
         gbs = alg / (ms * 1e-3) / 1e9
         out.append({"triangles": T, "device_ms": ms, "alg_bytes": alg, "achieved": gbs, "peak": peak,
                     "unit": "GB/s", "frac": gbs / peak, "peak_source": peak_kind})

@@ -267,7 +267,7 @@ GD_API gd_status gd_max_distance(gd_ctx *ctx, const gd_mesh *A, const gd_mesh *B
 /* Point-to-mesh distances (Eq. 1 with one side a single point; the 1-to-N
  * direction of Section 10's future work, with N query points): for each of
  * n world points, the closest point of mesh M placed by x (12 doubles, as
- * for the mesh queries).  Exact in float64: one thread per point walks M's
+ * for the mesh queries).  Exact in float64: one warp per point walks M's
  * tree once in float32 with a running bound that is always a true upper
  * bound (each triangle's float32 closest point, widened for the float32
  * errors), and takes the float64 distance of every triangle whose rigorous

@@ -3,8 +3,10 @@
 //
 // Phases (grid-wide barriers between them):
 //   0  per-query setup: B-local -> A-local rigid map in float64, its float32
-//      copy, and the absolute widening E of every float32 bound;
-//   1  the root pair enters the front (Algorithm 1, front initialisation);
+//      copy, and the absolute widening E of every float32 bound (a single query:
+//      by every CTA for itself);
+//   1  the root pair enters the front (Algorithm 1, front initialisation); a single
+//      query starts with the pairs two rounds of phase 2 would make of it;
 //   2  level loop (Algorithm 1's while loop, with the host round trip of the
 //      paper removed): the adaptive depth k is chosen on the device from the
 //      front length (Section 6), every entry is re-culled against the running
@@ -16,12 +18,14 @@
 //      bits (Section 7.4).  When the front first reaches a B subtree of 2^8
 //      leaves, that subtree is refit into A's frame (the paper refits B per
 //      frame, Section 8; here only the subtrees the front reaches are refit),
-//      and right after the first refit, greedy probes seed the bound;
+//      and greedy probes seed the bound: beside a single query's levels, in a
+//      batch right after the first refit;
 //   3  leaf-pair narrow phase: float32 triangle-triangle bounds, running bound
 //      update, candidate list;
 //   4  float64 refinement of the candidates in the world frame;
 //   5  witness selection (smallest original (tri_a, tri_b) at the extreme);
-//   6  witness points and result records.
+//   6  witness points and result records (a single query: 5 and 6 by CTA 0, which
+//      sends the record at once).
 #include <cfloat>
 #include <cstdio>
 #include <type_traits>
@@ -185,7 +189,7 @@ struct QView : QConst {
 // What a level of a batch reads of an entry's query: loaded for every entry (L1
 // hits) and not kept, since neighbouring entries belong to different queries
 // and a whole QView, refilled at every change, lived in local memory under the
-// batch's 64 registers.  The map itself is loaded only for pairs without a refit box.
+// batch's registers.  The map itself is loaded only for pairs without a refit box.
 struct BView {
     const QPack* k;
     const float* boxA;
