@@ -895,7 +895,9 @@ __device__ __forceinline__ bool line_apart(const CentreLine& c, float U, float E
 // running bound (*newU and *key are left as they are otherwise): 256 gear queries
 // 16.3 -> 14.0 ms.  TURN: with a refit box of B too, B's own box is tested along
 // that line; a flat patch that lies along B's axes is thin in that box and thick in
-// the refit one (leaf pairs of the gear batch 165 M -> 39 M, 14.0 -> 7.5 ms).
+// the refit one (leaf pairs of the gear batch 165 M -> 39 M, 14.0 -> 7.5 ms; of its
+// max form 77 M -> 9 M, 9.6 -> 5.3 ms; not for a single max query, whose levels
+// wait for the second box: rings 7.27 -> 7.68 ms).
 template <int KIND, bool FULL, bool LINE, bool TURN, class VT>
 __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
                                                 unsigned slot, float Ucur, bool* survive, unsigned* newU,
@@ -1658,7 +1660,7 @@ __device__ void expand_level(const AT& A, int level, unsigned n, int s, unsigned
             // (not for a single min query: its levels here are short, and the line
             // test's instructions cost the rings and spheres 0.5-0.8 us a level)
             constexpr bool kLine = KIND == 1 || !AT::kOne;
-            bound = pair_bounds<KIND, FULL, kLine, kLine && KIND == 0>(A, V, ia, ib, dBc, Ucur, &survive, &newU, &key);
+            bound = pair_bounds<KIND, FULL, kLine, kLine && (KIND == 0 || !AT::kOne)>(A, V, ia, ib, dBc, Ucur, &survive, &newU, &key);
         }
         warp_bound_update<KIND>(A, survive && newU != (KIND == 0 ? 0xffffffffu : 0u), q, newU);
         if (A.q_budget) {
@@ -1778,7 +1780,7 @@ __device__ void expand_level_entries(const AT& A, int level, unsigned n, unsigne
                 bool survive = false;
                 unsigned newU = KIND == 0 ? 0xffffffffu : 0u, key;
                 if (!one_root) slot = refit_slot(A, V, ib, dBc);
-                o[c].bound = pair_bounds_at<KIND, false, true, KIND == 0>(A, V, ia, ib, dBc, slot, Ucur, &survive, &newU, &key);
+                o[c].bound = pair_bounds_at<KIND, false, true, KIND == 0 || !AT::kOne>(A, V, ia, ib, dBc, slot, Ucur, &survive, &newU, &key);
                 if (survive) {
                     sm |= 1u << c;
                     best = KIND == 0 ? min(best, newU) : max(best, newU);
