@@ -138,7 +138,8 @@ typedef struct {
                               that run beside the traversal; batches: after
                               the first refit, at least one per query.  A min
                               query's repeated probes on fronts beyond 4 C use
-                              at least 256 */
+                              at least 256, a batch's beyond C / 2 one per warp
+                              of the launch */
     int64_t batch_budget;  /* batches: room per query and level in the first
                               round (default 2^23); a launch takes max_capacity
                               / (2 x budget) queries; half of the room is each

@@ -1171,7 +1171,8 @@ __device__ __forceinline__ bool wait_setup(const KArgs& A) {
 // the traversal's result does not depend on them.  They exist to reach a
 // near-final bound before the breadth-first levels widen (the sequential
 // depth-first behaviour Section 6 contrasts with).
-__device__ void setup_query_warp(const KArgs& A, int kind, bool state);
+template <class AT>
+__device__ void setup_query_warp(const AT& A, int q, int kind, bool state);
 
 template <int KIND, class AT>
 __device__ void probe(const AT& A, Item it, const QView& V) {
@@ -1271,7 +1272,7 @@ __device__ void probe_root(const AT& A, unsigned w, const QView& V) {
 template <int KIND, class AT>
 __device__ void bg_probe_cta(const AT& A) {
     __shared__ int s_ok;
-    if (threadIdx.x < 32) setup_query_warp(A, KIND, false);
+    if (threadIdx.x < 32) setup_query_warp(A, 0, KIND, false);
     __syncthreads();
     QView V;
     view(A, 0u, V);
@@ -1348,20 +1349,21 @@ __device__ __forceinline__ void setup_state(QState& s, int kind, unsigned slot_b
     s.pushed[0] = s.pushed[1] = 0u;
 }
 
-// The setup of a launch's only query by one warp (every lane calls it).  The
+// The setup of query q by one warp (every lane calls it).  The
 // nine entries of B's rotation in A's frame and the three of its translation
 // are independent three-term dot products of A's inverted 3x3 part with B's
 // transform, so lanes 0-8 compute one rotation entry each (row lane / 3,
 // column lane % 3) and lanes 9-11 one translation entry each.  A float64
-// instruction costs the same for one active lane as for a whole warp, and the
-// single thread of setup_query evaluating all twelve in turn spent
-// microseconds on them.  Lanes 0-8 also hold one entry of the adjugate each;
-// the determinant takes the first column from lanes 0, 3 and 6.  The constants
-// go to the CTA's copy, and in CTA 0 (state) to the query's state with the rest
-// of it.
-__device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
+// instruction costs the same for one active lane as for a whole warp: one thread
+// evaluating all twelve in turn took 3 us longer, and 256 queries of a batch, a
+// thread each, 57 us (a warp each, spread over the CTAs: 35).  Lanes 0-8 also hold one entry of the adjugate each;
+// the determinant takes the first column from lanes 0, 3 and 6.  A single query's
+// constants go to the CTA's copy, and in CTA 0 (state) to the query's state with
+// the rest of it; a batch query's to its state.
+template <class AT>
+__device__ void setup_query_warp(const AT& A, int q, int kind, bool state) {
     const int lane = threadIdx.x & 31;
-    QState& s = A.qs[0];
+    QState& s = A.qs[q];
     CtaState& cs = cta();
     const MeshDev* ma;
     const MeshDev* mb;
@@ -1369,9 +1371,9 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
     const double* xb;
     unsigned slot_base = 0;
     if (A.qin) {
-        ma = A.qin[0].A; mb = A.qin[0].B;
-        xa = A.qin[0].xa; xb = A.qin[0].xb;
-        slot_base = A.qin[0].slot_base;
+        ma = A.qin[q].A; mb = A.qin[q].B;
+        xa = A.qin[q].xa; xb = A.qin[q].xb;
+        slot_base = A.qin[q].slot_base;
     } else {
         ma = A.mA; mb = A.mB;
         xa = A.xa_src ? A.xa_src : A.xa_val;
@@ -1396,13 +1398,15 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
     const double r = i0 * v0 + i1 * v1 + i2 * v2;
     const float h = (float)r;
     const float lo = (float)(r - (double)h);
-    if (rot) {
+    if (AT::kOne && rot) {
         cs.v.X.R[lane] = h;
         cs.Rl[lane] = lo;
-    } else if (tra) {
+    } else if (AT::kOne && tra) {
         cs.v.X.t[i] = h;
         cs.tl[i] = lo;
     }
+    if (!AT::kOne && rot) s.pk.R[lane] = h;
+    else if (!AT::kOne && tra) s.pk.t[i] = h;
     if (state) {
         if (rot) {
             s.R[lane] = h;
@@ -1423,17 +1427,33 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
         // (every CTA's loads of the same two lines queue on them)
         const MeshDev da = A.host_desc ? A.dA : *ma, db = A.host_desc ? A.dB : *mb;
         const Widening E = setup_widening(da.P, db.P, tinf);
-        cs.v.E_box = E.E_box;
-        cs.v.E_tri = E.E_tri;
-        cs.E_df = E.E_df;
-        cs.v.boxA = da.box; cs.v.boxB = db.box;
-        cs.v.triA = da.tri; cs.v.triB = db.tri;
-        cs.v.TA = da.T; cs.v.TB = db.T;
-        cs.v.LA = da.L; cs.v.LB = db.L;
-        cs.v.dR = A.refit ? max(0, db.L - kRefitH) : -1;
-        cs.v.slot_base = slot_base;
-        cs.U = kind == 0 ? kFltMaxBits : 0u;
-        cs.stat = 0u;
+        if (AT::kOne) {
+            cs.v.E_box = E.E_box;
+            cs.v.E_tri = E.E_tri;
+            cs.E_df = E.E_df;
+            cs.v.boxA = da.box; cs.v.boxB = db.box;
+            cs.v.triA = da.tri; cs.v.triB = db.tri;
+            cs.v.TA = da.T; cs.v.TB = db.T;
+            cs.v.LA = da.L; cs.v.LB = db.L;
+            cs.v.dR = A.refit ? max(0, db.L - kRefitH) : -1;
+            cs.v.slot_base = slot_base;
+            cs.U = kind == 0 ? kFltMaxBits : 0u;
+            cs.stat = 0u;
+        } else {
+            QPack& k = s.pk;
+            k.E_box = E.E_box;
+            k.E_tri = E.E_tri;
+            k.LA = da.L;
+            k.LB = db.L;
+            k.dR = A.refit ? max(0, db.L - kRefitH) : -1;
+            k.boxA = da.box;
+            k.boxB = db.box;
+            k.slot_base = slot_base;
+            k.TA = (unsigned)da.T;
+            k.TB = (unsigned)db.T;
+            k.triA = da.tri;
+            k.triB = db.tri;
+        }
         if (state) {
             s.E_box = E.E_box;
             s.E_tri = E.E_tri;
@@ -1447,74 +1467,6 @@ __device__ void setup_query_warp(const KArgs& A, int kind, bool state) {
     // precedes the setup flag or the grid barrier
     if (state) __threadfence();
     __syncwarp();
-}
-
-__device__ void setup_query(const KArgs& A, int q, int kind) {
-    QState& s = A.qs[q];
-    const MeshDev* ma;
-    const MeshDev* mb;
-    const double* xa;
-    const double* xb;
-    unsigned slot_base = 0;
-    if (A.qin) {
-        ma = A.qin[q].A; mb = A.qin[q].B;
-        xa = A.qin[q].xa; xb = A.qin[q].xb;
-        slot_base = A.qin[q].slot_base;
-    } else {
-        ma = A.mA; mb = A.mB;
-        xa = A.xa_src ? A.xa_src : A.xa_val;
-        xb = A.xb_src ? A.xb_src : A.xb_val;
-    }
-    double Xa[12], Xb[12];
-    for (int i = 0; i < 12; ++i) { Xa[i] = xa[i]; Xb[i] = xb[i]; }
-    // inverse of A's 3x3 part (adjugate / determinant)
-    double a00 = Xa[0], a01 = Xa[1], a02 = Xa[2], a10 = Xa[4], a11 = Xa[5], a12 = Xa[6];
-    double a20 = Xa[8], a21 = Xa[9], a22 = Xa[10];
-    double c00 = a11 * a22 - a12 * a21, c01 = a02 * a21 - a01 * a22, c02 = a01 * a12 - a02 * a11;
-    double c10 = a12 * a20 - a10 * a22, c11 = a00 * a22 - a02 * a20, c12 = a02 * a10 - a00 * a12;
-    double c20 = a10 * a21 - a11 * a20, c21 = a01 * a20 - a00 * a21, c22 = a00 * a11 - a01 * a10;
-    double det = a00 * c00 + a01 * c10 + a02 * c20;
-    double id = 1.0 / det;
-    double Ai[9] = {c00 * id, c01 * id, c02 * id, c10 * id, c11 * id, c12 * id, c20 * id, c21 * id, c22 * id};
-    // R = Ai Rb, t = Ai (tb - ta)
-    double dt[3] = {Xb[3] - Xa[3], Xb[7] - Xa[7], Xb[11] - Xa[11]};
-    float tinf = 0.f;
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j) {
-            double r = Ai[3 * i] * Xb[j] + Ai[3 * i + 1] * Xb[4 + j] + Ai[3 * i + 2] * Xb[8 + j];
-            float h = (float)r;
-            s.R[3 * i + j] = h;
-            s.Rl[3 * i + j] = (float)(r - (double)h);
-        }
-        double tt = Ai[3 * i] * dt[0] + Ai[3 * i + 1] * dt[1] + Ai[3 * i + 2] * dt[2];
-        float h = (float)tt;
-        s.t[i] = h;
-        s.tl[i] = (float)(tt - (double)h);
-        tinf = fmaxf(tinf, fabsf(h));
-    }
-    const Widening E = setup_widening(ma->P, mb->P, tinf);
-    s.E_box = E.E_box;
-    s.E_tri = E.E_tri;
-    s.E_df = E.E_df;
-    s.A = ma;
-    s.B = mb;
-    for (int i = 0; i < 12; ++i) { s.xa[i] = Xa[i]; s.xb[i] = Xb[i]; }
-    setup_state(s, kind, slot_base, mb->L, A.refit);
-    QPack& k = s.pk;
-    k.E_box = E.E_box;
-    k.E_tri = E.E_tri;
-    k.LA = ma->L;
-    k.LB = mb->L;
-    k.dR = s.dR;
-    k.boxA = ma->box;
-    k.boxB = mb->box;
-    k.slot_base = slot_base;
-    k.TA = (unsigned)ma->T;
-    k.TB = (unsigned)mb->T;
-    k.triA = ma->tri;
-    k.triB = mb->tri;
-    for (int i = 0; i < 9; ++i) k.R[i] = s.R[i];
-    for (int i = 0; i < 3; ++i) k.t[i] = s.t[i];
 }
 
 // ------------------------------------------------------------- phase 2
@@ -2900,9 +2852,11 @@ __global__ void __launch_bounds__(kBlock, ONE ? 2 : GD_BATCH_CTAS) k_query(KArgs
         // (the two CTAs of an SM on different sub-partitions: float64 issues on
         // each one's own pipe)
         const unsigned sw = blockIdx.x == 0 || 2u * blockIdx.x < gridDim.x ? 0u : 1u;
-        if (threadIdx.x >> 5 == sw && (blockIdx.x == 0 || all_setup)) setup_query_warp(A, KIND, blockIdx.x == 0);
+        if (threadIdx.x >> 5 == sw && (blockIdx.x == 0 || all_setup)) setup_query_warp(A, 0, KIND, blockIdx.x == 0);
     } else {
-        for (int q = (int)gfirst; q < A.nq; q += (int)gstride) setup_query(A, q, KIND);
+        // a warp a query, spread over the CTAs
+        for (int q = (int)((threadIdx.x >> 5) * W + blockIdx.x); q < A.nq; q += (int)(W * (blockDim.x >> 5)))
+            setup_query_warp(A, q, KIND, true);
     }
     if (all_setup) {
         __syncthreads();
@@ -3006,18 +2960,24 @@ expand:
         // probes start where B's boxes are first exact in A's frame (or at
         // level 1 without refit), so that their greedy choices follow tight
         // boxes; the min kind probes again on every level whose front has
-        // outgrown 4x the work target, where the descents to leaves may also
-        // prove D_min = 0 and so stop the growth
-        const bool reprobe = KIND == 0 && probed && (long long)n >= 4 * A.work_target;
+        // outgrown 4x the work target (a batch: half of it), where the descents to
+        // leaves may also prove D_min = 0 and so stop the growth
+        const bool reprobe =
+            KIND == 0 && probed && (AT::kOne ? (long long)n >= 4 * A.work_target : 2 * (long long)n >= A.work_target);
         if (reprobe || (!probed && (A.refit ? ran : level == 1))) {
             probed = true;
             // greedy probes from entries spread evenly over the front: every
             // warp takes one (at least one per query when the grid allows)
             const unsigned nwarps = W * (blockDim.x >> 5);
-            const unsigned wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+            const unsigned wid = (threadIdx.x >> 5) * W + blockIdx.x;
             // (a min query's repeated probes on large fronts use at least
-            // kReprobes walks, enough to meet an intersection if there is one)
-            const unsigned want = max((unsigned)A.nq, reprobe ? max((unsigned)A.probes, kReprobes) : (unsigned)A.probes);
+            // kReprobes walks, enough to meet an intersection if there is one; a
+            // batch's a walk a warp, which takes as long: with 256 walks every level
+            // from 4x the target on, 256 gear queries, 48 of them intersecting,
+            // took 6.5 ms, with all warps 5.0, from half the target on 4.75)
+            const unsigned want = !AT::kOne && reprobe
+                                      ? nwarps
+                                      : max((unsigned)A.nq, reprobe ? max((unsigned)A.probes, kReprobes) : (unsigned)A.probes);
             const unsigned P = min(n, min(nwarps, want));
             const Item* in = (level & 1) ? A.front1 : A.front0;
             QView V;
