@@ -596,6 +596,36 @@ def test_device_resident_query(G, ctx, oracle_mod):
     G.gd_mesh_destroy(mb)
 
 
+@pytest.mark.parametrize("kind", ["min", "max"])
+def test_device_query_right_after_a_plain_call(G, ctx, oracle_mod, kind):
+    """A plain call returns with its record, before the launch's last bookkeeping: a
+    device query on another stream, and a plain call after that, share its counters
+    and must wait for them.  Two alternating placements, so that a stale answer shows."""
+    torch = pytest.importorskip("torch")
+    A, B, xa, xb = synth.config_tori(1)
+    xbs = [xb, np.asarray(xb, dtype=np.float64) + np.array([0, 0, 0, 0.25, 0, 0, 0, 0, 0, 0, 0, 0.0])]
+    ma, mb = _mesh(G, ctx, A), _mesh(G, ctx, B)
+    fn, k = (G.gd_min_distance, G.GD_MIN) if kind == "min" else (G.gd_max_distance, G.GD_MAX)
+    refs = [fn(ctx, ma, mb, xa, x) for x in xbs]
+    assert refs[0].d != refs[1].d
+    dxa = torch.tensor(xa, dtype=torch.float64, device="cuda")
+    dxb = [torch.tensor(x, dtype=torch.float64, device="cuda") for x in xbs]
+    out = torch.zeros(20, 10, dtype=torch.float64, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for i in range(20):
+        r = fn(ctx, ma, mb, xa, xbs[i & 1])
+        same_answer(r, refs[i & 1], oracle_mod, A, xa, B, xbs[i & 1], kind)
+        G.gd_query_device(ctx, ma, mb, k, dxa.data_ptr(), dxb[1 - (i & 1)].data_ptr(), out[i].data_ptr(),
+                          side.cuda_stream)
+        side.synchronize()
+    for i, raw in enumerate(out.cpu().numpy()):
+        same_answer(G.gd_result.from_buffer_copy(raw.tobytes()), refs[1 - (i & 1)], oracle_mod, A, xa, B,
+                    xbs[1 - (i & 1)], kind)
+    G.gd_mesh_destroy(ma)
+    G.gd_mesh_destroy(mb)
+
+
 def test_graph_replays_match_calls(G, ctx, oracle_mod):
     """A captured graph of one device-resident query, replayed after the
     transforms are updated in place, gives the answers of the synchronous
