@@ -239,11 +239,17 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const unsigned long 
     __shared__ unsigned long long s_key[kTile];
     __shared__ unsigned s_cnt[kSortWarps][256];
     __shared__ unsigned s_off[256];
-    __shared__ unsigned s_tile;
+    __shared__ unsigned s_tile, s_err;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_tile = atomicAdd(w.ticket + pass, 1u);
+    if (tid == 0) {
+        s_tile = atomicAdd(w.ticket + pass, 1u);
+        s_err = ld_relaxed(w.err);
+    }
     for (int k = 0; k < kSortWarps; ++k) s_cnt[k][tid] = 0u;
     __syncthreads();
+    // a wait of this pass or of one before it gave up: part of the input was never
+    // written, and its digits do not add up to the counts that place them
+    if (s_err) return;
     const unsigned tile = s_tile;
     const long long base = (long long)tile * kTile;
     const int m = (int)(n - base < kTile ? n - base : kTile);

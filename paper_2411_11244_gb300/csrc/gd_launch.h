@@ -43,7 +43,8 @@ struct BuildBuffers {
 // the index of the buffers that hold the sorted pairs.  Before it, sort_clear,
 // then a kernel that adds the keys' digits to w.hist (256 words a pass).
 // scratch: sort_scratch_bytes(n) bytes, 8-byte aligned.  A bounded wait that gave
-// up sets *w.err (device), and the sorted buffers are then not written.
+// up sets *w.err (device): the pass leaves the rest of its output as it was, the
+// passes after it do nothing, and nothing outside the buffers is written.
 size_t sort_scratch_bytes(long long n);
 SortWork sort_scratch(void* p, long long n);
 cudaError_t sort_clear(const SortWork& w, long long n, cudaStream_t stream);

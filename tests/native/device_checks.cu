@@ -1,0 +1,61 @@
+// Device code of the engine called beneath its C ABI, for the tests of what the
+// ABI cannot reach.  Compiled by the tests together with the sources it calls.
+#include <cuda_runtime.h>
+
+#include <vector>
+
+#include "gd_launch.h"
+
+namespace {
+struct Buffer {
+    void* p = nullptr;
+    explicit Buffer(size_t bytes) { cudaMalloc(&p, bytes); }
+    ~Buffer() { cudaFree(p); }
+};
+}  // namespace
+
+// A sort of n keys (the caller's; n and n + 4096 on one side of 2^18) whose first tile is never taken, so
+// that every other tile of the first pass waits for it until the wait gives up.
+// The buffers lie as the engine's do, keys, values and scratch in one allocation
+// with guard words behind it.  Returns 0, or
+// 1 a CUDA error, 2 no error word, 3 the input changed, 4 an output was written,
+// 5 a guard word was written.
+extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const unsigned long long* host, long long n,
+                                                                          int passes) {
+    using namespace gd;
+    constexpr unsigned long long kMark = 0x5aa5c33c5aa5c33cull;
+    // (tile numbers run from 1 on: room in the look-back table for one tile more)
+    const size_t k = (8 * (size_t)n + 255) / 256 * 256, v = (4 * (size_t)n + 255) / 256 * 256;
+    const size_t scratch = (sort_scratch_bytes(n + 4096) + 255) / 256 * 256, guard = 16 * (size_t)n + (1u << 20);
+    const size_t total = 2 * (k + v) + scratch + guard;
+    Buffer mem(total);
+    if (!mem.p) return 1;
+    std::vector<unsigned long long> all(total / 8, kMark);
+    cudaMemcpy(mem.p, all.data(), total, cudaMemcpyHostToDevice);
+    char* base = static_cast<char*>(mem.p);
+    unsigned long long* const keys[2] = {reinterpret_cast<unsigned long long*>(base),
+                                         reinterpret_cast<unsigned long long*>(base + k)};
+    unsigned* const vals[2] = {reinterpret_cast<unsigned*>(base + 2 * k), reinterpret_cast<unsigned*>(base + 2 * k + v)};
+    const SortWork w = sort_scratch(base + 2 * (k + v), n + 4096);
+    if (sort_clear(w, n + 4096, nullptr) != cudaSuccess) return 1;
+    std::vector<unsigned> hist(256 * passes, 0u);
+    for (long long i = 0; i < n; ++i)
+        for (int p = 0; p < passes; ++p) ++hist[256 * p + ((host[i] >> (8 * p)) & 255u)];
+    const unsigned one = 1u;
+    cudaMemcpy(keys[0], host, 8 * (size_t)n, cudaMemcpyHostToDevice);
+    cudaMemcpy(w.hist, hist.data(), sizeof(unsigned) * hist.size(), cudaMemcpyHostToDevice);
+    cudaMemcpy(w.ticket, &one, sizeof(one), cudaMemcpyHostToDevice);
+    radix_sort_pairs(w, keys, vals, n, 0, passes, nullptr);
+    unsigned err = 0;
+    cudaMemcpy(&err, w.err, sizeof(err), cudaMemcpyDeviceToHost);
+    cudaMemcpy(all.data(), mem.p, total, cudaMemcpyDeviceToHost);
+    if (cudaGetLastError() != cudaSuccess) return 1;
+    if (!err) return 2;
+    for (long long i = 0; i < n; ++i)
+        if (all[i] != host[i]) return 3;
+    for (size_t i = k / 8; i < 2 * (k + v) / 8; ++i)
+        if (all[i] != kMark) return 4;
+    for (size_t i = (total - guard) / 8; i < total / 8; ++i)
+        if (all[i] != kMark) return 5;
+    return 0;
+}
