@@ -228,6 +228,7 @@ long long table_entries(const gd_ctx* c, const gd_mesh* B) {
 
 gd_status ensure_table(gd_ctx* c, long long n) {
     if (n <= c->cap_table) return GD_OK;
+    ++c->ws_gen;  // graphs hold the table's address
     cudaFree(c->slot_of);
     c->slot_of = nullptr;
     c->cap_table = 0;
@@ -244,12 +245,12 @@ gd_status full_refit_tree(gd_ctx* c, const gd_mesh* B, KArgs& a) {
     if (c->tun.refit_mode != 3) return GD_OK;
     const long long nodes = 2ll << B->L;
     if (nodes > c->cap_ftree) {
+        ++c->ws_gen;  // (also where the allocation fails)
         cudaFree(c->ftree);
         c->ftree = nullptr;
         c->cap_ftree = 0;
         GD_CUDA(c, cudaMalloc(&c->ftree, sizeof(float) * 6 * nodes));
         c->cap_ftree = nodes;
-        ++c->ws_gen;
     }
     a.ftree = c->ftree;
     return GD_OK;

@@ -59,3 +59,23 @@ extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const 
         if (all[i] != kMark) return 5;
     return 0;
 }
+
+// Blocks of device memory filled with a byte, to lie where the engine has freed
+// some, and whether they still hold it.
+extern "C" __attribute__((visibility("default"))) void* check_block(size_t bytes, int value) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+    cudaMemset(p, value, bytes);
+    return p;
+}
+
+// 1: unchanged, 0: changed, -1: a CUDA error; frees it
+extern "C" __attribute__((visibility("default"))) int check_block_kept(void* p, size_t bytes, int value) {
+    std::vector<unsigned char> h(bytes);
+    cudaDeviceSynchronize();
+    if (cudaMemcpy(h.data(), p, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
+    cudaFree(p);
+    for (unsigned char c : h)
+        if (c != (unsigned char)value) return 0;
+    return 1;
+}

@@ -8,6 +8,8 @@ import subprocess
 import numpy as np
 import pytest
 
+from paper_2411_11244_gb300 import synth
+
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -20,7 +22,17 @@ def _compile(tmp, name, *defines):
     cmd = [B.nvcc(), *B.FLAGS, *B.ARCH, *defines, "-I", B.CSRC, "-shared", "-o", out, *src]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
-    return ctypes.CDLL(out)
+    lib = ctypes.CDLL(out)
+    lib.check_block.restype = ctypes.c_void_p
+    return lib
+
+
+@pytest.fixture(scope="module")
+def G():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2411_11244_gb300 import gdist
+    return gdist
 
 
 @pytest.fixture(scope="module")
@@ -37,3 +49,49 @@ def test_sort_that_gives_up_writes_nothing(checks, n):
     keys = rng.integers(0, 1 << 63, n, dtype=np.uint64)
     p = keys.ctypes.data_as(ctypes.c_void_p)
     assert checks.check_sort_gives_up(p, ctypes.c_longlong(n), 4) == 0
+
+
+def test_graph_after_a_batch_that_moves_the_refit_table(G, checks):
+    """The queues are at their limit, so a batch against a deep tree moves only
+    the table of refit roots (64 x 2^11 entries).  A graph made before is made
+    again by its next launch: it gives the plain call's answer, and what lies
+    where the table was stays as it is."""
+    torch = pytest.importorskip("torch")
+    ctx = G.gd_ctx_create(0)
+    try:
+        cap = 1 << 20
+        G.gd_ctx_set_tunables(ctx, front_capacity=cap, leaf_capacity=cap, cand_capacity=1 << 18, max_capacity=cap,
+                              batch_budget=cap >> 7)
+
+        def mesh(m):
+            h = G.gd_mesh_create(ctx, *m)
+            G.gd_bvh_build(h, ctx=ctx)
+            return h
+
+        a, small, deep = (mesh(m) for m in (synth.torus(1.0, 0.3, 40, 40), synth.geosphere(12, 0.5),
+                                            synth.geosphere(163, 0.5)))
+        assert G.gd_mesh_info(deep)[0] == 19
+        I = synth.identity_xform()
+        xs = [synth.xform(np.eye(3), (2.0 + 0.01 * i, 0.1, 0.2)) for i in range(64)]
+        G.gd_batch_query(ctx, G.make_queries([(a, small, I, x, G.GD_MIN) for x in xs]))
+        ref = G.gd_min_distance(ctx, a, small, I, xs[5])
+        dxa = torch.tensor(I, dtype=torch.float64, device="cuda")
+        dxb = torch.tensor(xs[5], dtype=torch.float64, device="cuda")
+        out = torch.zeros(10, dtype=torch.float64, device="cuda")
+        g = G.gd_graph_create(ctx, a, small, G.GD_MIN, dxa.data_ptr(), dxb.data_ptr(), out.data_ptr())
+        G.gd_batch_query(ctx, G.make_queries([(a, deep, I, x, G.GD_MIN) for x in xs]))
+        size = 4 << 16  # the table before the batch
+        blocks = [checks.check_block(ctypes.c_size_t(size), 0x5a) for _ in range(64)]
+        assert all(blocks)
+        torch.cuda.synchronize()
+        G.gd_graph_launch(g, None, ctx)
+        torch.cuda.synchronize()
+        r = G.gd_result.from_buffer_copy(out.cpu().numpy().tobytes())
+        kept = [checks.check_block_kept(ctypes.c_void_p(b), ctypes.c_size_t(size), 0x5a) for b in blocks]
+        assert kept == [1] * 64
+        assert (r.status, r.d, r.tri_a, r.tri_b) == (0, ref.d, ref.tri_a, ref.tri_b)
+        G.gd_graph_destroy(g)
+        for h in (a, small, deep):
+            G.gd_mesh_destroy(h)
+    finally:
+        G.gd_ctx_destroy(ctx)
