@@ -299,8 +299,9 @@ GD_API gd_status gd_naive_query(gd_ctx *ctx, const gd_mesh *A, const gd_mesh *B,
  * d_out a device pointer to one gd_result; stream is a cudaStream_t (NULL =
  * the context's stream).  Asynchronous (no host synchronisation); the
  * context's work buffers must already be sized (any prior synchronous query
- * does that).  Returns launch errors only; the per-query status is in
- * d_out->status. */
+ * does that).  stream may be under capture: the recorded launch uses the work
+ * buffers as they are then (capture again after a call that grew them).
+ * Returns launch errors only; the per-query status is in d_out->status. */
 GD_API gd_status gd_query_device(gd_ctx *ctx, const gd_mesh *A, const gd_mesh *B, gd_kind kind,
                                  const double *d_xa, const double *d_xb, gd_result *d_out, void *stream);
 /* Device-resident query that allocates nothing (the paper has no counterpart:

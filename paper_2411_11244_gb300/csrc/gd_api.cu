@@ -82,6 +82,7 @@ struct gd_ctx {
                                  // synchronous calls, [1..kPipe] for the server's pipelined launches
     unsigned long long hd_seq = 0;
     unsigned long long last_sync_seq = 0;  // the last synchronous query whose launch may still be leaving
+    bool captured = false;  // a caller's capture holds a launch that uses this context's buffers
     QState* qs = nullptr;
     QIn* qin_dev = nullptr;
     QIn* qin_host = nullptr;
@@ -373,11 +374,10 @@ int single_fuse_root(const gd_ctx* c, const gd_mesh* B) {
 }
 
 // A synchronous query returns when its record is there; its launch may still be
-// leaving, and resets the counters last.  Work for another stream that uses the
-// context's buffers waits for that (a few microseconds, without a CUDA call: the
-// caller's stream may be under capture).
-gd_status wait_left(gd_ctx* c, cudaStream_t st) {
-    if (st == c->stream || !c->hd || c->last_sync_seq == 0) return GD_OK;
+// leaving, and resets the counters last.  This waits until it has (a few
+// microseconds, without a CUDA call: a caller's stream may be under capture).
+gd_status wait_exit(gd_ctx* c) {
+    if (!c->hd || c->last_sync_seq == 0) return GD_OK;
     const volatile unsigned long long* left = &c->hd->exit_seq;
     const auto t0 = std::chrono::steady_clock::now();
     for (unsigned spin = 1; *left != c->last_sync_seq; ++spin) {
@@ -388,6 +388,16 @@ gd_status wait_left(gd_ctx* c, cudaStream_t st) {
     }
     c->last_sync_seq = 0;
     return GD_OK;
+}
+
+// Before work that uses the context's buffers goes to another stream.  In a
+// caller's capture that work is replayed without a call to this library, so from
+// the first such launch on a synchronous query itself returns only after its exit.
+gd_status wait_left(gd_ctx* c, cudaStream_t st) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) c->captured = true;
+    return st == c->stream ? GD_OK : wait_exit(c);
 }
 
 // CTAs of a single-query launch that run the traversal: the others (one per
@@ -511,9 +521,9 @@ gd_status run_single(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B, int kind, 
         int grid = grid_blocks(ctx, kind);
         a.work_ctas = single_work_ctas(ctx, grid);
         a.fuse_root = single_fuse_root(ctx, B);
-        // the launch's last CTA writes the result record to pinned host
-        // memory and stamps it with seq: no copy to enqueue and no stream
-        // synchronisation on the way back
+        // CTA 0 writes the result record to pinned host memory and stamps it with
+        // seq (the last CTA where the launch gave up): no copy to enqueue and no
+        // stream synchronisation on the way back.  The last CTA out stamps exit_seq
         const unsigned long long seq = ++ctx->hd_seq;
         a.host_done = ctx->hd;
         a.seq = seq;
@@ -537,9 +547,14 @@ gd_status run_single(gd_ctx* ctx, const gd_mesh* A, const gd_mesh* B, int kind, 
             std::memcpy(&r, (const void*)&ctx->hd->out, sizeof(r));
             last_abort = ctx->hd->last_abort;
             bad_index = ctx->hd->bad_index;
+            if (ctx->captured) {
+                s = wait_exit(ctx);
+                if (s != GD_OK) return s;
+            }
         } else {
             GD_CUDA(ctx, cudaMemcpyAsync(ctx->mb_host, ctx->mb_dev, kResultBytes, cudaMemcpyDeviceToHost, ctx->stream));
             GD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+            ctx->last_sync_seq = 0;
             r = ctx->mb_host->out;
             last_abort = ctx->mb_host->ctr[kCtrLastAbort];
             bad_index = ctx->mb_host->ctr[kCtrBadIndex];

@@ -626,6 +626,40 @@ def test_device_query_right_after_a_plain_call(G, ctx, oracle_mod, kind):
     G.gd_mesh_destroy(mb)
 
 
+def test_callers_capture_replayed_right_after_a_plain_call(G, ctx, oracle_mod):
+    """A device query in a caller's own CUDA graph is replayed without a call to the
+    library that could wait for the plain call before it: that call returns only once
+    its launch has reset the counters they share."""
+    torch = pytest.importorskip("torch")
+    A, B, xa, xb = synth.config_tori(1)
+    xb = [np.asarray(xb, dtype=np.float64), np.asarray(xb, dtype=np.float64) + np.array([0, 0, 0, 0.25, 0, 0, 0, 0, 0, 0, 0, 0])]
+    ma, mb = _mesh(G, ctx, A), _mesh(G, ctx, B)
+    refs = [G.gd_min_distance(ctx, ma, mb, xa, x) for x in xb]
+    assert refs[0].d != refs[1].d
+    dxa = torch.tensor(xa, dtype=torch.float64, device="cuda")
+    dxb = torch.tensor(xb[1], dtype=torch.float64, device="cuda")
+    out = torch.zeros(10, dtype=torch.float64, device="cuda")
+    rows = torch.zeros(100, 10, dtype=torch.float64, device="cuda")
+    side = torch.cuda.Stream()
+    own = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(own, stream=side):
+        G.gd_query_device(ctx, ma, mb, G.GD_MIN, dxa.data_ptr(), dxb.data_ptr(), out.data_ptr(), side.cuda_stream)
+    plain = []
+    with torch.cuda.stream(side):
+        for i in range(len(rows)):
+            plain.append(G.gd_min_distance(ctx, ma, mb, xa, xb[0]))
+            own.replay()
+            rows[i].copy_(out)
+            side.synchronize()
+    for r in plain:
+        same_answer(r, refs[0], oracle_mod, A, xa, B, xb[0], "min")
+    for raw in rows.cpu().numpy():
+        same_answer(G.gd_result.from_buffer_copy(raw.tobytes()), refs[1], oracle_mod, A, xa, B, xb[1], "min")
+    G.gd_mesh_destroy(ma)
+    G.gd_mesh_destroy(mb)
+
+
 def test_graph_replays_match_calls(G, ctx, oracle_mod):
     """A captured graph of one device-resident query, replayed after the
     transforms are updated in place, gives the answers of the synchronous
