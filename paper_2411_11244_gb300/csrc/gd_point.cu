@@ -147,7 +147,10 @@ __device__ __forceinline__ void tri_bounds_sq(const V3<float>* w, float e, float
         mag = fmaxf(mag, aq.x * fabsf(w[k].x) + aq.y * fabsf(w[k].y) + aq.z * fabsf(w[k].z));
     }
     const float num = smin - mag * 0x1p-22f - (aq.x + aq.y + aq.z) * (X * 0x1p-22f + e);
-    *lower = num > 0.f && qq > 0.f ? num * num / qq * (1.f - 0x1p-20f) : 0.f;
+    // (num * num leaves float32's range at a distance of 4e9, where num and qq are
+    // still far inside it: an infinite bound would drop the nearest triangle.  Below
+    // 1e-15 the terms' own roundings are no longer relative)
+    *lower = num > 0.f && qq > 0x1p-100f ? num / qq * num * (1.f - 0x1p-20f) : 0.f;
 }
 
 // Whether the plane across the direction to the triangle's centroid keeps it

@@ -1130,6 +1130,31 @@ def test_point_ties_take_the_smallest_index(G, ctx, oracle_mod, copies):
         G.gd_mesh_destroy(h)
 
 
+@pytest.mark.parametrize("far", [4e9, 5e9, 1e12, 1e18, 3e19, 1e-12, 1e-17])
+def test_point_distances_near_the_ends_of_float32(G, ctx, oracle_mod, far):
+    """Points so far from a mesh that a float32 distance to the fourth power
+    overflows, so far that its square does, and points so near that they underflow."""
+    rng = np.random.default_rng(77)
+    m = synth.torus(1.0, 0.3, 40, 25)
+    h = _mesh(G, ctx, m)
+    try:
+        I = synth.identity_xform()
+        d = rng.normal(size=(33, 3))
+        d *= far / np.linalg.norm(d, axis=1)[:, None]
+        pts = d if far > 1 else m[0][rng.integers(0, len(m[0]), len(d))].astype(np.float64) + d
+        r = G.gd_point_distance(ctx, h, I, pts)
+        if far < 1e15:
+            check_points(r, m, I, pts, oracle_mod)
+        else:
+            # (the oracle's plane projection cancels to nothing out there.)  The mesh lies within 1.31 of the
+            # origin, and three float64 squares, their sum and its root are off by at most 4 units in the last place
+            n = np.linalg.norm(pts, axis=1)
+            assert (r["status"] == 0).all()
+            assert (np.abs(r["d"] - n) <= 1.31 + 8 * 2.0 ** -53 * n).all()
+    finally:
+        G.gd_mesh_destroy(h)
+
+
 def test_point_order_and_caller_order_agree(G, ctx):
     """Calls of 2^14 points and more are walked along a Morton curve; the same
     points in small calls are not: the records are the same bits."""
