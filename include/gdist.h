@@ -222,7 +222,9 @@ GD_API gd_status gd_mesh_create(gd_ctx *ctx, const float *verts, int64_t nv, con
  * leaves (L = floor(log2 nt)) of one or two consecutive sorted triangles, leaf
  * boxes that are exact bounds of their vertices, and a level-by-level union of
  * boxes up to the root.  Every box is tight (Section 4, tightness lemma).
- * Synchronous.  GD_ERR_INVALID_ARG on bad indices or non-finite vertices. */
+ * Synchronous.  GD_ERR_INVALID_ARG on bad indices or non-finite vertices;
+ * GD_ERR_TIMEOUT if a tile of the sort waited longer than the context's
+ * timeout_ns for the tiles before it (the mesh is then unbuilt). */
 GD_API gd_status gd_bvh_build(gd_mesh *mesh, const gd_build_opts *opts);
 /* Deformable meshes (Section 8: the BVH is refit on the fly when vertices
  * move).  Replaces the vertex positions of a built mesh (same count nv, same

@@ -186,7 +186,7 @@ cudaError_t sort_buffers(gd_ctx* c, long long n, SortBuffers* b) {
         b->keys[i] = reinterpret_cast<unsigned long long*>(c->sort_mem + i * k);
         b->vals[i] = reinterpret_cast<unsigned*>(c->sort_mem + 2 * k + i * v);
     }
-    b->work = sort_scratch(c->sort_mem + 2 * (k + v), n);
+    b->work = sort_scratch(c->sort_mem + 2 * (k + v), n, (unsigned long long)c->tun.timeout_ns);
     return cudaSuccess;
 }
 

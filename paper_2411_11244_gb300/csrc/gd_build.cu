@@ -22,7 +22,6 @@ constexpr int kSortWarps = kSortThreads / 32;
 // that they spread over the SMs (a tile's ranking is a chain over its items)
 constexpr int kItemsSmall = 4, kItemsLarge = 16;
 constexpr long long kSmallSort = 1 << 18;
-constexpr unsigned long long kSortTimeout = 2000000000ull;  // ns a tile waits for its predecessors
 
 // float -> uint32 whose unsigned order is the float order
 __device__ __forceinline__ unsigned ordered(float f) {
@@ -328,7 +327,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_pass(const unsigned long 
                 if ((spin & 255u) == 0u) {
                     const unsigned long long now = globaltimer();
                     if (t0 == 0) t0 = now;
-                    if (now - t0 > kSortTimeout || ld_relaxed(w.err)) {
+                    if (now - t0 > w.timeout_ns || ld_relaxed(w.err)) {
                         atomicExch(w.err, 1u);
                         failed = true;
                         break;
@@ -615,13 +614,14 @@ size_t sort_scratch_bytes(long long n) {
     return 256 * sizeof(unsigned long long) * tiles + sizeof(unsigned) * (256 * kSortPasses + 64);
 }
 
-SortWork sort_scratch(void* p, long long n) {
+SortWork sort_scratch(void* p, long long n, unsigned long long timeout_ns) {
     const size_t words = (sort_scratch_bytes(n) - sizeof(unsigned) * (256 * kSortPasses + 64)) / sizeof(unsigned long long);
     SortWork w;
     w.status = static_cast<unsigned long long*>(p);
     w.hist = reinterpret_cast<unsigned*>(w.status + words);
     w.ticket = w.hist + 256 * kSortPasses;
     w.err = w.ticket + 32;
+    w.timeout_ns = timeout_ns;
     return w;
 }
 

@@ -17,6 +17,7 @@ struct SortWork {
     unsigned* hist;              // digit counts, 256 a pass
     unsigned* ticket;            // next tile of each pass
     unsigned* err;               // a wait gave up
+    unsigned long long timeout_ns;  // a tile's longest wait for one before it
 };
 
 struct BuildBuffers {
@@ -46,7 +47,7 @@ struct BuildBuffers {
 // up sets *w.err (device): the pass leaves the rest of its output as it was, the
 // passes after it do nothing, and nothing outside the buffers is written.
 size_t sort_scratch_bytes(long long n);
-SortWork sort_scratch(void* p, long long n);
+SortWork sort_scratch(void* p, long long n, unsigned long long timeout_ns);
 cudaError_t sort_clear(const SortWork& w, long long n, cudaStream_t stream);
 int radix_sort_pairs(const SortWork& w, unsigned long long* const keys[2], unsigned* const vals[2], long long n,
                      int lo_bit, int passes, cudaStream_t stream);

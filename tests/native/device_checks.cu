@@ -2,9 +2,12 @@
 // ABI cannot reach.  Compiled by the tests together with the sources it calls.
 #include <cuda_runtime.h>
 
+#include <chrono>
 #include <vector>
 
 #include "gd_launch.h"
+
+#define EXPORT extern "C" __attribute__((visibility("default")))
 
 namespace {
 struct Buffer {
@@ -14,14 +17,14 @@ struct Buffer {
 };
 }  // namespace
 
-// A sort of n keys (the caller's; n and n + 4096 on one side of 2^18) whose first tile is never taken, so
-// that every other tile of the first pass waits for it until the wait gives up.
-// The buffers lie as the engine's do, keys, values and scratch in one allocation
-// with guard words behind it.  Returns 0, or
-// 1 a CUDA error, 2 no error word, 3 the input changed, 4 an output was written,
+// A sort of n keys (the caller's; n and n + 4096 on one side of 2^18) whose first
+// tile is never taken, so that every other tile of the first pass waits for it
+// until the wait gives up, after timeout_ns.  The buffers lie as the engine's do,
+// keys, values and scratch in one allocation with guard words behind it.  *ms: how
+// long the sort took.  Returns 0, or 1 a CUDA error, 2 no error word, 3 the input changed, 4 an output was written,
 // 5 a guard word was written.
-extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const unsigned long long* host, long long n,
-                                                                          int passes) {
+EXPORT int check_sort_gives_up(const unsigned long long* host, long long n, int passes, unsigned long long timeout_ns,
+                               double* ms) {
     using namespace gd;
     constexpr unsigned long long kMark = 0x5aa5c33c5aa5c33cull;
     // (tile numbers run from 1 on: room in the look-back table for one tile more)
@@ -36,7 +39,7 @@ extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const 
     unsigned long long* const keys[2] = {reinterpret_cast<unsigned long long*>(base),
                                          reinterpret_cast<unsigned long long*>(base + k)};
     unsigned* const vals[2] = {reinterpret_cast<unsigned*>(base + 2 * k), reinterpret_cast<unsigned*>(base + 2 * k + v)};
-    const SortWork w = sort_scratch(base + 2 * (k + v), n + 4096);
+    const SortWork w = sort_scratch(base + 2 * (k + v), n + 4096, timeout_ns);
     if (sort_clear(w, n + 4096, nullptr) != cudaSuccess) return 1;
     std::vector<unsigned> hist(256 * passes, 0u);
     for (long long i = 0; i < n; ++i)
@@ -45,7 +48,11 @@ extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const 
     cudaMemcpy(keys[0], host, 8 * (size_t)n, cudaMemcpyHostToDevice);
     cudaMemcpy(w.hist, hist.data(), sizeof(unsigned) * hist.size(), cudaMemcpyHostToDevice);
     cudaMemcpy(w.ticket, &one, sizeof(one), cudaMemcpyHostToDevice);
+    cudaDeviceSynchronize();
+    const auto t0 = std::chrono::steady_clock::now();
     radix_sort_pairs(w, keys, vals, n, 0, passes, nullptr);
+    cudaDeviceSynchronize();
+    *ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     unsigned err = 0;
     cudaMemcpy(&err, w.err, sizeof(err), cudaMemcpyDeviceToHost);
     cudaMemcpy(all.data(), mem.p, total, cudaMemcpyDeviceToHost);
@@ -62,7 +69,7 @@ extern "C" __attribute__((visibility("default"))) int check_sort_gives_up(const 
 
 // Blocks of device memory filled with a byte, to lie where the engine has freed
 // some, and whether they still hold it.
-extern "C" __attribute__((visibility("default"))) void* check_block(size_t bytes, int value) {
+EXPORT void* check_block(size_t bytes, int value) {
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
     cudaMemset(p, value, bytes);
@@ -70,7 +77,7 @@ extern "C" __attribute__((visibility("default"))) void* check_block(size_t bytes
 }
 
 // 1: unchanged, 0: changed, -1: a CUDA error; frees it
-extern "C" __attribute__((visibility("default"))) int check_block_kept(void* p, size_t bytes, int value) {
+EXPORT int check_block_kept(void* p, size_t bytes, int value) {
     std::vector<unsigned char> h(bytes);
     cudaDeviceSynchronize();
     if (cudaMemcpy(h.data(), p, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;

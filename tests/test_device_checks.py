@@ -44,11 +44,15 @@ def checks(tmp_path_factory):
 def test_sort_that_gives_up_writes_nothing(checks, n):
     """A tile of the first pass never publishes: the waits for it run out, the
     passes that follow leave their buffers alone (the pairs that the first pass
-    did not write would be placed beyond them), and the error word is set."""
+    did not write would be placed beyond them), and the error word is set.  The
+    waits end after the limit that the sort was given: 2 ms here, and far less than
+    the 2 s of a context's default with the launches around them."""
     rng = np.random.default_rng(n)
     keys = rng.integers(0, 1 << 63, n, dtype=np.uint64)
     p = keys.ctypes.data_as(ctypes.c_void_p)
-    assert checks.check_sort_gives_up(p, ctypes.c_longlong(n), 4) == 0
+    ms = ctypes.c_double()
+    assert checks.check_sort_gives_up(p, ctypes.c_longlong(n), 4, ctypes.c_ulonglong(2_000_000), ctypes.byref(ms)) == 0
+    assert 2.0 <= ms.value < 500.0
 
 
 def test_graph_after_a_batch_that_moves_the_refit_table(G, checks):
