@@ -897,7 +897,8 @@ __device__ __forceinline__ bool line_apart(const CentreLine& c, float U, float E
 // that line; a flat patch that lies along B's axes is thin in that box and thick in
 // the refit one (leaf pairs of the gear batch 165 M -> 39 M, 14.0 -> 7.5 ms; of its
 // max form 77 M -> 9 M, 9.6 -> 5.3 ms; not for a single max query, whose levels
-// wait for the second box: rings 7.27 -> 7.68 ms).
+// wait for the second box: rings 7.27 -> 7.68 ms).  Conventional bounds only (the
+// ablation) take none of it: its pairs are culled by their conventional bound alone.
 template <int KIND, bool FULL, bool LINE, bool TURN, class VT>
 __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, unsigned ia, unsigned ib, int db,
                                                 unsigned slot, float Ucur, bool* survive, unsigned* newU,
@@ -912,7 +913,7 @@ __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, uns
         Box bb = FULL ? load_box_cg(A.ftree, ib) : load_box_cg(A.rbox, refit_index(V, slot, ib, db));
         bound = KIND == 0 ? lower_min_sq(ba, bb.lo, bb.hi) : upper_max_sq(ba, bb.lo, bb.hi);
         *survive = KIND == 0 ? bound <= min_keep_threshold(Ucur, V.E_box) : bound >= max_keep_threshold(Ucur, V.E_box);
-        if (LINE) {
+        if (LINE && !A.conventional) {
             if (!*survive) return bound;
             if (TURN && line_apart<KIND>(centre_line<false>(map_of(V), ba, b0), Ucur, tri_widening(V))) {
                 *survive = false;
@@ -938,7 +939,7 @@ __device__ __forceinline__ float pair_bounds_at(const KArgs& A, const VT& V, uns
         enclose(X, bb, elo, ehi);
         bound = KIND == 0 ? lower_min_sq(ba, elo, ehi) : upper_max_sq(ba, elo, ehi);
         *survive = KIND == 0 ? bound <= min_keep_threshold(Ucur, V.E_box) : bound >= max_keep_threshold(Ucur, V.E_box);
-        if (LINE) {
+        if (LINE && !A.conventional) {
             if (!*survive) return bound;
             const CentreLine c = centre_line<false>(X, ba, bb);
             if (line_apart<KIND>(c, Ucur, tri_widening(V))) *survive = false;

@@ -463,6 +463,58 @@ def test_conventional_bounds_ablation(G, oracle_mod):
         G.gd_ctx_destroy(c)
 
 
+@pytest.mark.parametrize("kind", ["min", "max"])
+@pytest.mark.parametrize("entry", ["call", "batch"])
+def test_conventional_bounds_cull_by_boxes_alone(G, oracle_mod, kind, entry):
+    """bounds_mode 2 culls a pair by its conventional bound only, the gap of A's box
+    and the box around B's turned one (max: their farthest points): every leaf pair
+    whose bound is within the answer gets to the leaf phase, however far apart its
+    turned boxes are.  Parallel flat patches, A's turned against its own axes and B's
+    not, so that B's boxes are thin as they lie and thick when enclosed; the bounds of
+    all leaf pairs in float64 against the engine's count."""
+    c = G.gd_ctx_create(0)
+    try:
+        rng = np.random.default_rng(83)
+        Q = synth.random_rotation(rng)
+        A, B = _plate(24, 0.0), _plate(25, 0.0)
+        A = ((A[0] @ Q.T).astype(np.float32), A[1])
+        ma, mb = _mesh(G, c, A), _mesh(G, c, B)
+        G.gd_ctx_set_tunables(c, bounds_mode=2, refit_mode=2)
+        k = G.GD_MIN if kind == "min" else G.GD_MAX
+        R = Q @ synth.rot_axis((0, 0, 1), 0.4)
+        xa = synth.identity_xform()
+        xs = [synth.xform(R, R[:, 2] * h) for h in ((0.2, 0.25, 0.3) if kind == "min" else (50.0, 80.0, 100.0))]
+        boxes = []
+        for h, x in ((ma, np.eye(3, 4)), (mb, np.asarray(xs[0]).reshape(3, 4))):
+            leaf = G.gd_mesh_download(h)[0]
+            leaf = leaf[len(leaf) // 2:].astype(np.float64)
+            m, e = (leaf[:, 3:] + leaf[:, :3]) / 2, (leaf[:, 3:] - leaf[:, :3]) / 2
+            boxes.append((m @ x[:, :3].T, e @ np.abs(x[:, :3]).T))
+        want = 0
+        got = 0
+        for x in xs:
+            t = np.asarray(x).reshape(3, 4)[:, 3]
+            d = np.abs(boxes[0][0][:, None] - (boxes[1][0] + t)[None])
+            e = boxes[0][1][:, None] + boxes[1][1][None]
+            ref = oracle_mod.bvh_query(oracle_mod.Bvh(A), xa, oracle_mod.Bvh(B), x, kind).d
+            if kind == "min":
+                want += (np.linalg.norm(np.maximum(d - e, 0), axis=2) < ref * (1 - 1e-5)).sum()
+            else:
+                want += (np.linalg.norm(d + e, axis=2) > ref * (1 + 1e-5)).sum()
+        if entry == "batch":
+            assert all(r.status == 0 for r in G.gd_batch_query(c, [(ma, mb, xa, x, k) for x in xs]))
+            got = G.gd_get_stats(c)["leaf_pairs"]
+        else:
+            for x in xs:
+                assert (G.gd_min_distance if kind == "min" else G.gd_max_distance)(c, ma, mb, xa, x).status == 0
+                got += G.gd_get_stats(c)["leaf_pairs"]
+        assert got >= want > 0
+        G.gd_mesh_destroy(ma)
+        G.gd_mesh_destroy(mb)
+    finally:
+        G.gd_ctx_destroy(c)
+
+
 def test_autotune_keeps_answers(G, oracle_mod):
     """gd_autotune picks tunables by timing and never changes an answer: the
     answers before and after tuning are the same (single query and batch)."""
