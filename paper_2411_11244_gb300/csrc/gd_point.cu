@@ -600,7 +600,9 @@ __device__ __forceinline__ unsigned walk(const PointArgs& g, PointWarp& W, unsig
 // entries of the warp's list, join the slot's chain (thinned to kPartCands by
 // float64 if need be).  The last part of the point gathers the chain into the
 // list and returns the number of candidates it is left with (kNone if a part
-// ran into the deadline); any other returns 0.
+// ran into the deadline); any other returns 0.  Its float64 distances go to the
+// call's count at once (a counter of the caller's, reached through a pointer, cost
+// 8 % of a large call: the caller then holds it in memory).
 __device__ __noinline__ unsigned join_part(const PointArgs& g, PointWarp& W, unsigned i, unsigned slot, unsigned n0,
                                            unsigned nc) {
     const unsigned lane = threadIdx.x & 31, lt = lanemask_lt();
@@ -613,6 +615,7 @@ __device__ __noinline__ unsigned join_part(const PointArgs& g, PointWarp& W, uns
             int id;
             V3<double> q;
             exact_candidates(g, W, n0, nc, &d2, &id, &q);
+            if (lane == 0) atomicAdd(g.ws + kPointExact, (unsigned long long)nc);
             const unsigned win = nearest_lane(d2, id);
             const unsigned j = W.cj[n0 + win];
             const float low = W.clow[n0 + win];
@@ -672,6 +675,7 @@ __device__ __noinline__ unsigned join_part(const PointArgs& g, PointWarp& W, uns
         __syncwarp();
         if (n > 32u) {
             U = fminf(U, thin_candidates(g, W, n0 + n));
+            if (lane == 0) atomicAdd(g.ws + kPointExact, 32ull);
             n -= 31u;
         }
         k = __shfl_sync(kFull, __ldcg(&p.next), 0);

@@ -1207,6 +1207,22 @@ def test_point_distances_near_the_ends_of_float32(G, ctx, oracle_mod, far):
         G.gd_mesh_destroy(h)
 
 
+def test_point_stats_count_every_exact_distance(G, ctx):
+    """Copies of one triangle: no float32 bound tells them apart, so each of them
+    takes a float64 distance for each point, whatever part of a divided walk meets it."""
+    T, n = 1 << 14, 24
+    v = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0]], dtype=np.float32)
+    m = (v, np.tile(np.array([[0, 1, 2]], dtype=np.int32), (T, 1)))
+    h = _mesh(G, ctx, m)
+    try:
+        pts = np.random.default_rng(5).uniform(0.5, 2.0, (n, 3))
+        r = G.gd_point_distance(ctx, h, synth.identity_xform(), pts)
+        assert (r["status"] == 0).all() and (r["tri"] == 0).all()
+        assert G.gd_point_stats(ctx)["exact_tests"] >= n * T
+    finally:
+        G.gd_mesh_destroy(h)
+
+
 def test_point_order_and_caller_order_agree(G, ctx):
     """Calls of 2^14 points and more are walked along a Morton curve; the same
     points in small calls are not: the records are the same bits."""
