@@ -189,7 +189,13 @@ typedef struct {
 /* ---- context ----------------------------------------------------------- */
 
 /* Create a context on CUDA device `device`; allocates its stream and, on the
- * first query, its work buffers.  GD_ERR_CUDA if the device is unusable. */
+ * first query, its work buffers.  GD_ERR_CUDA if the device is unusable.
+ * Device memory that a context keeps from one call to the next, besides its
+ * meshes and the queues of gd_tunables: up to 256 MB of what destroyed meshes
+ * leave; the scratch of its largest sort (24 to 26 bytes a triangle or point),
+ * as long as that is below 1 GiB; 14 MB from the first point query on, and
+ * copies of host points and results (72 bytes a point of the largest call).
+ * gd_ctx_destroy gives everything back. */
 GD_API gd_status gd_ctx_create(int device, gd_ctx **out);
 GD_API void gd_ctx_destroy(gd_ctx *ctx);
 /* Message of the last failing call on ctx ("" if none).  Owned by ctx. */
@@ -241,6 +247,8 @@ GD_API gd_status gd_bvh_build(gd_mesh *mesh, const gd_build_opts *opts);
  * nv differs from the mesh's or a coordinate is not finite (the mesh is then
  * left unbuilt until the next successful update or build). */
 GD_API gd_status gd_mesh_update(gd_mesh *mesh, const float *verts, int64_t nv);
+/* Waits for the device, then frees the mesh: of its memory at most 256 MB stay
+ * with the context for its next meshes (see gd_ctx_create). */
 GD_API void gd_mesh_destroy(gd_mesh *mesh);
 /* Device time in ms of the kernels of the mesh's last gd_bvh_build (index
  * validation, Morton codes, radix sort, leaves and level reduction; CUDA

@@ -159,6 +159,19 @@ void mesh_free(gd_ctx* c, T* p) {
     if (p) cudaFreeAsync(p, c->stream);
 }
 
+// Gives back what the pool holds beyond its live meshes and kPoolKeep.  (The pool's
+// own release threshold counts the live ones too, and acts at the next
+// synchronisation, whenever that is: it is off.)
+void trim_pool(gd_ctx* c) {
+    unsigned long long held = 0, used = 0;
+    if (cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+        return;
+    if (held <= used + kPoolKeep) return;
+    cudaStreamSynchronize(c->stream);  // the frees are done when the stream has passed them
+    cudaMemPoolTrimTo(c->pool, used + kPoolKeep);
+}
+
 // Buffers of a sort of n keys.  One allocation a context, reused by its builds
 // and point queries, which all run on its stream; above kSortKeep it is given
 // back at the end of the call (drop_sort), so that one huge mesh does not hold it.
@@ -672,7 +685,7 @@ GD_API gd_status gd_ctx_create(int device, gd_ctx** out) {
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = device;
-    unsigned long long keep = kPoolKeep;
+    unsigned long long keep = ~0ull;  // (trim_pool bounds it)
     if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
         cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
         if (c->pool) cudaMemPoolDestroy(c->pool);
@@ -1001,6 +1014,7 @@ GD_API void gd_mesh_destroy(gd_mesh* m) {
     mesh_free(c, m->d_order);
     mesh_free(c, m->d_stris);
     cudaFree(m->d_desc);
+    trim_pool(c);
     delete m;
 }
 

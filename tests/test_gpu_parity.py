@@ -226,6 +226,32 @@ def test_bvh_build_equal_keys(G, ctx, case, bits):
         G.gd_mesh_destroy(h)
 
 
+def test_mesh_destroy_gives_memory_back(G):
+    """Free device memory after large meshes are destroyed: what it was, less the
+    256 MB of mesh buffers and the sort scratch that a context says it keeps."""
+    torch = pytest.importorskip("torch")
+    c = G.gd_ctx_create(0)
+    try:
+        G.gd_mesh_destroy(_mesh(G, c, synth.torus(1.0, 0.3, 32, 32)))
+        m = synth.torus(1.0, 0.3, 2000, 1100)
+        T = len(m[1])
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        for live in (0, 1):
+            hs = [_mesh(G, c, m) for _ in range(2 + live)]
+            held = before - torch.cuda.mem_get_info()[0]
+            assert held > len(hs) * 82 * T  # (vertices, indices, records, order, boxes)
+            for h in hs[live:]:
+                G.gd_mesh_destroy(h)
+            kept = before - torch.cuda.mem_get_info()[0]
+            # (a mesh that is left, and 32 blocks of 2 MB of rounding)
+            assert kept <= live * held // len(hs) + (256 << 20) + 25 * T + (64 << 20)
+        G.gd_mesh_destroy(hs[0])
+    finally:
+        G.gd_ctx_destroy(c)
+    assert before - torch.cuda.mem_get_info()[0] <= 64 << 20
+
+
 def test_bvh_build_rejects_bad_input(G, ctx):
     v = np.zeros((3, 3), np.float32)
     t = np.array([[0, 1, 3]], np.int32)
