@@ -336,7 +336,8 @@ def build_roofline(G, meshes, peak, peak_kind):
     written each; the first reads no values), the order within equal keys (12 B/T
     read, 4 B/T written), leaves (4 B/T order + 12 B/T indices + 12 B/V read,
     48 B/T triangle records and 12 B/T vertex indices in leaf order, for the
-    refits, written) and 24 B per node box written."""
+    refits, written) and 24 B per node box written.  (The ring has no run of
+    equal codes that would have it sorted a second time on all bits.)"""
     out = []
     for h, T, V in meshes:
         L, _ = G.gd_mesh_info(h)

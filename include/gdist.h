@@ -252,7 +252,9 @@ GD_API gd_status gd_mesh_update(gd_mesh *mesh, const float *verts, int64_t nv);
 GD_API void gd_mesh_destroy(gd_mesh *mesh);
 /* Device time in ms of the kernels of the mesh's last gd_bvh_build (index
  * validation, Morton codes, radix sort, leaves and level reduction; CUDA
- * events on the context's stream around them, allocations excluded).
+ * events on the context's stream around them, allocations excluded).  A mesh
+ * with more than 128 triangles of one shortened Morton code is sorted and built
+ * a second time on all bits, and both count.
  * Preprocessing: the paper times its builds apart from the queries (Section
  * 8).  GD_ERR_NOT_BUILT for a mesh without a tree. */
 GD_API gd_status gd_mesh_build_time(const gd_mesh *mesh, double *device_ms);

@@ -952,13 +952,13 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     m->h_desc.L = L;
     m->h_desc.P = 0.f;  // (the root's kernel writes the device's)
     GD_CUDA(ctx, cudaMemcpyAsync(m->d_desc, &m->h_desc, sizeof(MeshDev), cudaMemcpyHostToDevice, ctx->stream));
-    // device time of the build's kernels: events around them, on the stream they run on
+    // device time of the build's kernels: events around them, on the stream they run
+    // on; a second build on all bits adds its own, not the read-back in between
     unsigned flags[16];
+    float build_ms = 0.f;
     for (int all_bits = 0; all_bits < 2; ++all_bits) {
-        if (!all_bits) {
-            cudaEventRecord(ctx->build_ev[0], ctx->stream);
-            e = build_validate(b, ctx->stream);
-        }
+        cudaEventRecord(ctx->build_ev[0], ctx->stream);
+        if (!all_bits) e = build_validate(b, ctx->stream);
         if (e == cudaSuccess) e = build_tree(b, all_bits != 0, desc_P(m), ctx->stream);
         cudaEventRecord(ctx->build_ev[1], ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(flags, b.flags, sizeof(flags), cudaMemcpyDeviceToHost, ctx->stream);
@@ -967,10 +967,12 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
         if (flags[0]) return fail(ctx, GD_ERR_INVALID_ARG, "triangle index out of range");
         if (flags[1]) return fail(ctx, GD_ERR_INVALID_ARG, "non-finite vertex coordinate");
         if (flags[kFlagSort]) return fail(ctx, GD_ERR_TIMEOUT, "a device-side wait of the build's sort timed out");
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, ctx->build_ev[0], ctx->build_ev[1]);
+        build_ms += ms;
         if (!flags[kFlagTies]) break;
     }
-    m->build_ms = 0.f;
-    cudaEventElapsedTime(&m->build_ms, ctx->build_ev[0], ctx->build_ev[1]);
+    m->build_ms = build_ms;
     m->h_desc.P = root_P(flags);
     m->L = L;
     m->built = true;
