@@ -698,10 +698,15 @@ def test_device_resident_query(G, ctx, oracle_mod):
 
 
 @pytest.mark.parametrize("kind", ["min", "max"])
-def test_device_query_right_after_a_plain_call(G, ctx, oracle_mod, kind):
+@pytest.mark.parametrize("entry", ["query", "graph"])
+def test_device_query_right_after_a_plain_call(G, ctx, oracle_mod, kind, entry):
     """A plain call returns with its record, before the launch's last bookkeeping: a
-    device query on another stream, and a plain call after that, share its counters
-    and must wait for them.  Two alternating placements, so that a stale answer shows."""
+    device query or a graph's launch on another stream, and a plain call after that,
+    share its counters and must wait for them.  Two alternating placements, so that a
+    stale answer shows; both calls go straight to the library, one after the other,
+    as the launch is gone a few microseconds after its record (counted once: 1,581 of
+    1,600 such calls found it still there)."""
+    import ctypes
     torch = pytest.importorskip("torch")
     A, B, xa, xb = synth.config_tori(1)
     xbs = [xb, np.asarray(xb, dtype=np.float64) + np.array([0, 0, 0, 0.25, 0, 0, 0, 0, 0, 0, 0, 0.0])]
@@ -709,20 +714,38 @@ def test_device_query_right_after_a_plain_call(G, ctx, oracle_mod, kind):
     fn, k = (G.gd_min_distance, G.GD_MIN) if kind == "min" else (G.gd_max_distance, G.GD_MAX)
     refs = [fn(ctx, ma, mb, xa, x) for x in xbs]
     assert refs[0].d != refs[1].d
+    n = 400
     dxa = torch.tensor(xa, dtype=torch.float64, device="cuda")
     dxb = [torch.tensor(x, dtype=torch.float64, device="cuda") for x in xbs]
-    out = torch.zeros(20, 10, dtype=torch.float64, device="cuda")
+    one = torch.zeros(10, dtype=torch.float64, device="cuda")
+    out = torch.zeros(n, 10, dtype=torch.float64, device="cuda")
     side = torch.cuda.Stream()
+    st = side.cuda_stream
+    lib = G.load()
+    plain = lib.gd_min_distance if kind == "min" else lib.gd_max_distance
+    device = lib.gd_graph_launch if entry == "graph" else lib.gd_query_device
+    graphs = [G.gd_graph_create(ctx, ma, mb, k, dxa.data_ptr(), d.data_ptr(), one.data_ptr()) for d in dxb]
+    if entry == "graph":
+        args = [(graphs[1 - i % 2], st) for i in range(n)]
+    else:
+        args = [(ctx, ma, mb, k, dxa.data_ptr(), dxb[1 - i % 2].data_ptr(), one.data_ptr(), st) for i in range(n)]
+    hxa, *hxb = [(ctypes.c_double * 12)(*x) for x in (xa, *xbs)]
+    rec = [G.gd_result() for _ in range(n)]
+    ok = True
     torch.cuda.synchronize()
-    for i in range(20):
-        r = fn(ctx, ma, mb, xa, xbs[i & 1])
-        same_answer(r, refs[i & 1], oracle_mod, A, xa, B, xbs[i & 1], kind)
-        G.gd_query_device(ctx, ma, mb, k, dxa.data_ptr(), dxb[1 - (i & 1)].data_ptr(), out[i].data_ptr(),
-                          side.cuda_stream)
-        side.synchronize()
+    with torch.cuda.stream(side):
+        for i in range(n):
+            r1 = plain(ctx, ma, mb, hxa, hxb[i % 2], rec[i])
+            r2 = device(*args[i])
+            ok = ok and r1 == r2 == G.GD_OK
+            out[i].copy_(one)
+            side.synchronize()
+    assert ok
     for i, raw in enumerate(out.cpu().numpy()):
-        same_answer(G.gd_result.from_buffer_copy(raw.tobytes()), refs[1 - (i & 1)], oracle_mod, A, xa, B,
-                    xbs[1 - (i & 1)], kind)
+        for r, x in ((rec[i], i % 2), (G.gd_result.from_buffer_copy(raw.tobytes()), 1 - i % 2)):
+            same_answer(r, refs[x], oracle_mod, A, xa, B, xbs[x], kind)
+    for g in graphs:
+        G.gd_graph_destroy(g)
     G.gd_mesh_destroy(ma)
     G.gd_mesh_destroy(mb)
 
