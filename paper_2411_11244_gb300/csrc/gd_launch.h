@@ -111,9 +111,13 @@ enum : int {
 
 // Shared walks: a warp with a long walk gives parts of its stack to idle
 // warps.  Fixed room, reused by every call; when it is full walks are no longer
-// divided.
-constexpr unsigned kPointMaxSlots = 1u << 14;   // points with a shared walk
-constexpr unsigned kPointMaxShares = 1u << 16;  // gifts
+// divided.  (The tests compile it with little room too.)
+#ifndef GD_POINT_SLOTS
+#define GD_POINT_SLOTS (1u << 14)
+#define GD_POINT_SHARES (1u << 16)
+#endif
+constexpr unsigned kPointMaxSlots = GD_POINT_SLOTS;    // points with a shared walk
+constexpr unsigned kPointMaxShares = GD_POINT_SHARES;  // gifts
 
 struct PointSlot {
     unsigned U;       // least upper bound of all parts (float bits, squared)

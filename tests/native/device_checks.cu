@@ -67,6 +67,61 @@ EXPORT int check_sort_gives_up(const unsigned long long* host, long long n, int 
     return 0;
 }
 
+// Point queries on a mesh, twice over with the same room for shared walks: out
+// (2 n records) and the counters of the second call.  Returns 0, or 1 on an error.
+EXPORT int check_points(const float* verts, long long nv, const int32_t* tris, long long nt, const double* points,
+                        long long n, gd_point_result* out, unsigned long long* slots, unsigned long long* gifts,
+                        unsigned long long* parts) {
+    using namespace gd;
+    int L = 0;
+    while ((2ll << L) <= nt) ++L;
+    Buffer v(12 * (size_t)nv), t(12 * (size_t)nt), box(24 * (2ull << L)), tri(48 * (size_t)nt), order(4 * (size_t)nt),
+        stris(12 * (size_t)nt), flags(64), P(4), k0(8 * (size_t)nt), k1(8 * (size_t)nt), v0(4 * (size_t)nt),
+        v1(4 * (size_t)nt), scratch(sort_scratch_bytes(nt)), pts(24 * (size_t)n), res(sizeof(gd_point_result) * n),
+        ws(8 * kPointWords), share(kPointShareBytes);
+    cudaMemcpy(v.p, verts, 12 * (size_t)nv, cudaMemcpyHostToDevice);
+    cudaMemcpy(t.p, tris, 12 * (size_t)nt, cudaMemcpyHostToDevice);
+    cudaMemcpy(pts.p, points, 24 * (size_t)n, cudaMemcpyHostToDevice);
+    cudaMemset(share.p, 0, kPointShareBytes);
+    BuildBuffers b{};
+    b.verts = static_cast<float*>(v.p); b.tris = static_cast<int32_t*>(t.p); b.nv = nv; b.nt = nt; b.L = L;
+    b.morton_bits = 21;
+    b.box = static_cast<float*>(box.p); b.tri = static_cast<float4*>(tri.p);
+    b.order = static_cast<unsigned*>(order.p); b.stris = static_cast<int32_t*>(stris.p);
+    b.flags = static_cast<unsigned*>(flags.p);
+    b.keys[0] = static_cast<unsigned long long*>(k0.p); b.keys[1] = static_cast<unsigned long long*>(k1.p);
+    b.vals[0] = static_cast<unsigned*>(v0.p); b.vals[1] = static_cast<unsigned*>(v1.p);
+    b.sort = sort_scratch(scratch.p, nt, 2000000000ull);
+    if (build_validate(b, nullptr) != cudaSuccess || build_tree(b, true, static_cast<float*>(P.p), nullptr) != cudaSuccess)
+        return 1;
+    PointArgs g{};
+    g.box = b.box; g.tri = b.tri; g.T = nt; g.L = L;
+    g.x[0] = g.x[5] = g.x[10] = 1.0;
+    g.pts = static_cast<double*>(pts.p);
+    g.n = n;
+    g.out = static_cast<gd_point_result*>(res.p);
+    g.ws = static_cast<unsigned long long*>(ws.p);
+    g.timeout_ns = 2000000000ll;
+    g.shares = static_cast<PointShare*>(share.p);
+    g.parts = reinterpret_cast<PointPart*>(g.shares + kPointMaxShares);
+    g.slots = reinterpret_cast<PointSlot*>(g.parts + kPointMaxSlots + kPointMaxShares);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
+    unsigned long long w[kPointWords];
+    for (unsigned call = 0; call < 2; ++call) {
+        g.epoch = call + 1;
+        cudaMemset(res.p, 0xff, sizeof(gd_point_result) * n);
+        if (launch_point(g, sms, nullptr) != cudaSuccess) return 1;
+        cudaMemcpy(out + call * n, res.p, sizeof(gd_point_result) * n, cudaMemcpyDeviceToHost);
+        cudaMemcpy(w, ws.p, sizeof(w), cudaMemcpyDeviceToHost);
+        if (w[kPointTimeout] || w[kPointAnswered] != (unsigned long long)n) return 1;
+    }
+    *slots = w[kPointSlots];
+    *gifts = w[kPointTail];
+    *parts = w[kPointParts];
+    return cudaDeviceSynchronize() == cudaSuccess ? 0 : 1;
+}
+
 // Blocks of device memory filled with a byte, to lie where the engine has freed
 // some, and whether they still hold it.
 EXPORT void* check_block(size_t bytes, int value) {

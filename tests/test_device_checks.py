@@ -18,7 +18,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 def _compile(tmp, name, *defines):
     from paper_2411_11244_gb300 import build as B
     out = os.path.join(tmp, name + ".so")
-    src = [os.path.join(HERE, "native", "device_checks.cu"), os.path.join(B.CSRC, "gd_build.cu")]
+    src = [os.path.join(HERE, "native", "device_checks.cu"), os.path.join(B.CSRC, "gd_build.cu"),
+           os.path.join(B.CSRC, "gd_point.cu")]
     cmd = [B.nvcc(), *B.FLAGS, *B.ARCH, *defines, "-I", B.CSRC, "-shared", "-o", out, *src]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
@@ -99,3 +100,43 @@ def test_graph_after_a_batch_that_moves_the_refit_table(G, checks):
             G.gd_mesh_destroy(h)
     finally:
         G.gd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("room", [None, (3, 9), (2, 64), (64, 2)])
+def test_points_with_shared_walks(G, tmp_path, checks, room):
+    """Points around the centre of a sphere, whose walks meet all of it: warps give
+    parts of them away, as the counters show, also when there is too little room for
+    the points that want to share or for their gifts, and in a second call over the
+    first one's records.  Every answer is that of the same point in a call by itself
+    (and of gd_point_distance for all of them)."""
+    lib = checks
+    if room:
+        lib = _compile(str(tmp_path), "room", f"-DGD_POINT_SLOTS={room[0]}u", f"-DGD_POINT_SHARES={room[1]}u")
+    v, t = synth.geosphere(64, 1.0, 1e-4, 3)
+    n = 200
+    pts = np.random.default_rng(9).normal(0.0, 1e-3, (n, 3))
+    out = (G.gd_point_result * (2 * n))()
+    c = [ctypes.c_ulonglong() for _ in range(3)]
+    p = [a.ctypes.data_as(ctypes.c_void_p) for a in (v, t, pts)]
+    assert lib.check_points(p[0], ctypes.c_longlong(len(v)), p[1], ctypes.c_longlong(len(t)), p[2],
+                            ctypes.c_longlong(n), out, *map(ctypes.byref, c)) == 0
+    slots, gifts, parts = (x.value for x in c)
+    if room is None:
+        assert slots > 0 and gifts > slots and parts > 0
+    else:
+        assert slots > room[0] or gifts > room[1]
+    ctx = G.gd_ctx_create(0)
+    try:
+        h = G.gd_mesh_create(ctx, v, t)
+        G.gd_bvh_build(h, ctx=ctx)
+        ref = G.gd_point_distance(ctx, h, synth.identity_xform(), pts)
+        for i in (0, 7, n - 1):
+            one = G.gd_point_distance(ctx, h, synth.identity_xform(), pts[i:i + 1])
+            assert one.tobytes() == ref[i:i + 1].tobytes()
+        G.gd_mesh_destroy(h)
+    finally:
+        G.gd_ctx_destroy(ctx)
+    assert (ref["status"] == 0).all()
+    got = np.frombuffer(out, dtype=ref.dtype)
+    for f in ("d", "tri", "p", "status"):
+        assert np.array_equal(got[f][:n], ref[f]) and np.array_equal(got[f][n:], ref[f])
