@@ -16,15 +16,16 @@
 // distance, so the answer is the exact minimum over all triangles, the
 // smallest original index among ties.
 //
-// What bounds it: issue slots and L1/L2 latency of the box tests (about 4,000
-// a point on a ring, most of them near-ties), not the bytes of the points.
+// What bounds it: issue slots and L1/L2 latency of the box tests (3,200 a point
+// around a ring on average, most of them near-ties), not the bytes of the points.
 // A thread per point, with float64 in the walk, left one lane of a warp
 // working at a time: 262,144 device points against a 7.5 M-triangle ring took
 // 258 ms, 1,000 host points against a 204,800-triangle gear 9.4 ms; one warp
-// per point alone 18.8 ms and 0.49 ms (one walk of 500 K tests, with its
-// neighbours, ran half of that alone); with long walks divided among idle warps
-// 9.6 ms (8.7 until the points run out) and 0.20 ms.  20, 24 and 28 warps an SM
-// took 11.5, 10.9 and 10.4 ms at one stage of this, 32 (with 64 registers) 12.0.
+// per point alone 13.6 ms (18.8 for another draw of the points, in which one
+// walk of 500 K tests, with its neighbours, ran for half of that) and 0.29 ms;
+// with long walks divided among idle warps 9.8 and 0.15 ms.  20, 24 and 28 warps
+// an SM took 11.5, 10.9 and 10.4 ms at one stage of this, 32 (with 64 registers)
+// 12.0.
 #include <algorithm>
 #include <cfloat>
 #include <cstdint>

@@ -43,6 +43,13 @@ constexpr unsigned kFltMaxBits = 0x7f7fffffu;
 constexpr unsigned kNoSlot = 0xffffffffu, kClaimed = 0xfffffffeu;
 constexpr unsigned kReprobes = 256;
 constexpr int kDryRunDepth = 30;  // L_A + L_B from which background CTAs warm the code of later phases
+// L_A + L_B from which the two levels after start_level take two levels a side at
+// most.  Plain calls on spheres, rings, tori and gears of 2^11 to 2^18 leaves each,
+// limited against free: at 22 and 24 up to 6 us slower (min 59 against 53); at 26
+// to 32 within 3.3 us either way; at 34 faster (spheres 79 against 82, tori 109
+// against 113, max 182 against 189, gears 119 against 130, max 105 against 119); at
+// 36 up to 7 us faster.
+constexpr int kDeepStart = 30;
 
 // ------------------------------------------------------------- thresholds
 // All float32 bounds are made rigorous for float64 world distances:
@@ -662,9 +669,9 @@ __device__ __forceinline__ void tri_pair_bounds_tight(const AT& A, unsigned q, c
                                                       const Tri32& TB, float* lo, float* up) {
     const V3<float> o = TA.v[0];
     if constexpr (GROUP) {
-        // B's nine coordinates over the group's lanes (lane 0 also takes the last),
-        // in a loop: a ninth of the instructions, which a query's first pairs wait
-        // for as they are fetched (leaf phase of two tori 9.8 -> 8.7 us)
+        // B's nine coordinates: a lane each of the first eight, then every lane the
+        // ninth, in a loop: a ninth of the instructions, which a query's first pairs
+        // wait for as they are fetched (leaf phase of two tori 9.8 -> 8.7 us)
         const CtaState& c = cta();
         const unsigned sub = threadIdx.x & 7u, first = threadIdx.x & 24u;
         float mine[2];
@@ -1148,8 +1155,8 @@ __device__ __noinline__ void certify_zero(const AT& A, unsigned q, unsigned ta, 
     }
 }
 
-// A background CTA's wait (bounded) until the query's state is set up; called by
-// one thread.  False if the launch was aborted.
+// A background CTA's wait (bounded) until the query's state is set up, by one
+// thread or a whole warp.  False if the launch was aborted.
 __device__ __forceinline__ bool wait_setup(const KArgs& A) {
     const unsigned long long t0 = globaltimer();
     while (!ld_acquire(A.ctr + kCtrSetupDone)) {
@@ -3006,9 +3013,9 @@ expand:
         int k = adaptive_k(n, A.work_target, A.k_max);
         // The two levels after start_level run before the probes' bound is there;
         // on deep trees they go two levels a side at most, since what they keep
-        // under a loose bound multiplies below (icospheres: 200 -> 191 us max,
-        // 116 -> 111 min; trees of 11 levels lost 4 us to the extra level)
-        if (AT::kOne && start && level <= 2 && cta().v.LA + cta().v.LB >= kDryRunDepth) k = min(k, 2);
+        // under a loose bound multiplies below (icospheres of 1.3 M triangles:
+        // 200 -> 191 us max, 116 -> 111 min)
+        if (AT::kOne && start && level <= 2 && cta().v.LA + cta().v.LB >= kDeepStart) k = min(k, 2);
         int s = min(2 * k, (int)rmax);
         if (s < 1) s = 1;
         if (lead) {
