@@ -144,8 +144,8 @@ gd_status cuda_fail(gd_ctx* ctx, cudaError_t e, const char* where) {
 // bytes of what destroyed meshes leave (cudaMalloc and cudaFree map and unmap
 // whatever exceeds 1 MB on every call: 0.1 ms and more each).  The memory is
 // allocated and freed in the order of the context's stream; the calls that make a
-// mesh synchronise that stream before they return, and gd_mesh_destroy the
-// device before it frees.
+// mesh synchronise that stream before they return, and gd_mesh_destroy waits for
+// the device before it frees.
 constexpr unsigned long long kPoolKeep = 256ull << 20;
 
 template <class T>
@@ -157,6 +157,15 @@ cudaError_t mesh_alloc(gd_ctx* c, T** p, size_t bytes) {
 template <class T>
 void mesh_free(gd_ctx* c, T* p) {
     if (p) cudaFreeAsync(p, c->stream);
+}
+
+// Waits for the work of all streams, as cudaFree does.  (cudaDeviceSynchronize is
+// refused while any stream is being captured, in a relaxed mode or on another
+// thread too, and that capture is lost with it.)
+cudaError_t wait_device() {
+    void* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, 256);
+    return e == cudaSuccess ? cudaFree(p) : e;
 }
 
 // Gives back what the pool holds beyond its live meshes and kPoolKeep.  (The pool's
@@ -925,7 +934,7 @@ GD_API gd_status gd_bvh_build(gd_mesh* m, const gd_build_opts* opts) {
     int L = 0;
     while ((2ll << L) <= m->nt) ++L;
     // a tree that work on any stream may still read is only overwritten once that is done
-    if (m->d_desc) GD_CUDA(ctx, cudaDeviceSynchronize());
+    if (m->d_desc) GD_CUDA(ctx, wait_device());
     m->built = false;
     m->tree = false;
     BuildBuffers b{};
@@ -1008,14 +1017,13 @@ GD_API void gd_mesh_destroy(gd_mesh* m) {
     if (!m) return;
     gd_ctx* c = m->ctx;
     cudaSetDevice(c->device);
-    cudaDeviceSynchronize();  // queries on any stream
+    cudaFree(m->d_desc);  // waits for queries on any stream (a mesh without it has had none), as wait_device does
     mesh_free(c, m->d_verts);
     mesh_free(c, m->d_tris);
     mesh_free(c, m->d_box);
     mesh_free(c, m->d_tri);
     mesh_free(c, m->d_order);
     mesh_free(c, m->d_stris);
-    cudaFree(m->d_desc);
     trim_pool(c);
     delete m;
 }

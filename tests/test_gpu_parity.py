@@ -249,6 +249,73 @@ def test_build_time_of_a_repeated_build_is_its_kernels(G, ctx):
     assert rest[1] > 1.4 * rest[0], rest
 
 
+@pytest.mark.parametrize("mode", ["relaxed", "thread_local"])
+def test_mesh_calls_beside_a_capture(G, mode):
+    """Meshes are made, built again, updated and destroyed while another stream is
+    being captured (on this thread in relaxed mode, or on another one): the calls
+    work, and the capture goes on."""
+    import threading
+    torch = pytest.importorskip("torch")
+    c = G.gd_ctx_create(0)
+    I, X = synth.identity_xform(), synth.xform(np.eye(3), (3, 0, 0))
+    m = synth.torus(1.0, 0.3, 40, 40)
+    a, b = _mesh(G, c, m), _mesh(G, c, m)
+    ref = G.gd_min_distance(c, a, b, I, X)
+    errors = []
+
+    def calls():
+        try:
+            d = _mesh(G, c, m)
+            G.gd_mesh_update(d, m[0], c)
+            assert G.gd_min_distance(c, a, d, I, X).d == ref.d
+            G.gd_mesh_destroy(d)
+            G.gd_bvh_build(a, ctx=c)
+            assert G.gd_min_distance(c, a, b, I, X).d == ref.d
+        except Exception as e:
+            errors.append(e)
+
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream(), capture_error_mode=mode):
+        x.add_(1)
+        if mode == "relaxed":
+            calls()
+        else:
+            t = threading.Thread(target=calls)
+            t.start()
+            t.join()
+        x.add_(1)
+    g.replay()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert (x == 2).all()
+    G.gd_mesh_destroy(a)
+    G.gd_mesh_destroy(b)
+    G.gd_ctx_destroy(c)
+
+
+@pytest.mark.parametrize("call", ["destroy", "rebuild"])
+def test_mesh_calls_wait_for_other_streams(G, ctx, call):
+    """A mesh may still be read by work on any stream when it is destroyed or built
+    again: the call returns after that work."""
+    torch = pytest.importorskip("torch")
+    h = _mesh(G, ctx, synth.torus(1.0, 0.3, 40, 40))
+    side, ev = torch.cuda.Stream(), torch.cuda.Event()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(40_000_000)  # about 20 ms
+        ev.record()
+    assert not ev.query()
+    if call == "destroy":
+        G.gd_mesh_destroy(h)
+    else:
+        G.gd_bvh_build(h, ctx=ctx)
+    assert ev.query()
+    if call == "rebuild":
+        G.gd_mesh_destroy(h)
+
+
 def test_mesh_destroy_gives_memory_back(G):
     """Free device memory after large meshes are destroyed: what it was, less the
     256 MB of mesh buffers and the sort scratch that a context says it keeps."""
