@@ -176,7 +176,8 @@ typedef struct {
     uint32_t phase_ns[12];       /* device time of: setup, subtree refits, probes,
                                     all levels, leaf narrow phase, float64
                                     refinement, wait for the refinement of the
-                                    other CTAs, witness selection, result
+                                    other CTAs, witness selection (a single
+                                    query: 0, with the records), result
                                     records, total, (2 unused); CTA 0's view;
                                     after gd_batch_query, summed over its
                                     launches */
@@ -269,9 +270,9 @@ GD_API gd_status gd_mesh_download(const gd_mesh *mesh, float *boxes, int32_t *tr
 
 /* Minimum distance D_min (Eq. 1).  xa, xb: host transforms.  Synchronous:
  * the transforms travel as launch parameters, one persistent traversal
- * launch runs, and its last CTA writes the result record to the context's
- * pinned host memory, which the call waits for (bounded by the launch's own
- * completion; no stream synchronisation on the way back). */
+ * launch runs and writes the result record to the context's pinned host
+ * memory as soon as it is final, which the call waits for (bounded by the
+ * launch's own completion; no stream synchronisation on the way back). */
 GD_API gd_status gd_min_distance(gd_ctx *ctx, const gd_mesh *A, const gd_mesh *B, const double xa[12],
                                  const double xb[12], gd_result *out);
 /* Maximum distance D_max (Eq. 2); same contract as gd_min_distance. */
